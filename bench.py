@@ -392,8 +392,7 @@ def frame_stream(hsc, f, dev, args, world, F, fp32_rate, fp32_peak_note, with_e2
     tune = {"config": tune_cfg, "seconds": time.perf_counter() - t0,
             "how": "hsc_autotune on the first cube: Gram TMA staging depth {3, 4} (B <= 128), "
                    "projection/SVM {1, 4} pixels per thread x {2, 4, 8, 16} CTAs per SM, pruned "
-                   "KNN walk {32 px x 8, 32 x 6, 32 x 12, 64 x 8, and 32 x 8 and 64 x 8 with "
-                   "the window tile staged by TMA} (pixels per CTA x undecided keys per lane), "
+                   "KNN walk {4, 1, 2, 8, 4, 6} warps per CTA, "
                    "median of 3 runs each; results do not depend on them"}
     streams = [stream] + [torch.cuda.Stream(dev) for _ in range(F - 1)]
     ctxs = [ctx] + [hsc.Context(dev.index or 0, stream=s) for s in streams[1:]]
@@ -492,10 +491,8 @@ def frame_stream(hsc, f, dev, args, world, F, fp32_rate, fp32_peak_note, with_e2
     ctx.sync()
     full_ms_launch = full_ms["knn"] / n_full
     heap_ms_launch = heap_ms["knn"] / n_heap
-    # ---- the pruned walk's variants (the autotuner's candidates; 4 and 5
-    # stage the window tile with one TMA box instead of 16-byte asynchronous
-    # copies): the KNN stage of the profiled steps per variant, then the tuned
-    # variant again
+    # ---- the pruned walk's variants (the autotuner's candidates): the KNN
+    # stage of the profiled steps per variant, then the tuned variant again
     walk_ms = {}
     for v in range(6):
         ctx.set_tuning(B, H, W, k, (tune_cfg["gram_stages"], tune_cfg["svm_px"],
@@ -505,9 +502,8 @@ def frame_stream(hsc, f, dev, args, world, F, fp32_rate, fp32_peak_note, with_e2
     ctx.set_tuning(B, H, W, k, (tune_cfg["gram_stages"], tune_cfg["svm_px"],
                                 tune_cfg["svm_blocks_per_sm"], tune_cfg["knn_variant"]))
     knn_walks = {"ms_per_launch": {("%d: %s" % (v, name)): round(walk_ms[v], 5)
-                                   for v, name in enumerate(("32 px x 8 keys", "32 x 6", "32 x 12",
-                                                             "64 x 8", "32 x 8, TMA tile",
-                                                             "64 x 8, TMA tile"))},
+                                   for v, name in enumerate(("4 warps", "1 warp", "2 warps", "8 warps",
+                                                             "4 warps", "6 warps"))},
                  "tuned": tune_cfg["knn_variant"],
                  "note": "the KNN stage (pruned walk + redo pass) of the profiled steps per walk "
                          "variant; the outputs are the same bit for bit"}

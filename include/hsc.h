@@ -363,18 +363,15 @@ hsc_status hsc_pca_diagnostics(hsc_ctx *ctx, int32_t *sweeps, int32_t *refine_it
  * candidates of the tensor-core Gram's TMA staging depth (3 or 4 stages;
  * B <= 128), of the projection/SVM pass's launch shape (1 or 4 pixels per
  * thread x 2, 4, 8 or 16 CTAs per SM) and, given KNN parameters with
- * lambda > 0 and the pruned search, of the pruned walk's pixels per CTA and
- * undecided keys per lane (variants 0: 32 and 8, 1: 32 and 6, 2: 32 and 12,
- * 3: 64 and 8; 4 and 5: 0 and 3 with each CTA's window tile staged by one
- * TMA box, where the map allows a tensor map; every pixel's neighbour
+ * lambda > 0 and the pruned search, of the pruned walk's warps per CTA
+ * (variants 0: 4, 1: 1, 2: 2, 3: 8, 4: 4, 5: 6; every pixel's neighbour
  * probabilities are added in one
  * canonical order whichever pass completes it, so O is the same) on this cube
  * and model (median of 3 runs each, CUDA events on the context's stream,
  * which it synchronises), and keeps the fastest for frames of this shape (B,
  * H*W, n_classes) in the context: hsc_classify, hsc_classify_batch and
  * hsc_pca_one_band use it for frames of that shape, the defaults for others
- * (the walk: variant 4, which takes variant 0's copies where the map does not
- * allow a tensor map).
+ * (the walk: variant 4).
  * Retuning replaces it.
  *   params  KNN parameters (nullable: the walk is not tuned)
  *   config  4 int32 (host, nullable): stages, pixels per thread, CTAs per SM,
@@ -396,12 +393,14 @@ hsc_status hsc_set_tuning(hsc_ctx *ctx, int B, int H, int W, int n_classes,
 hsc_status hsc_measure_fma_rate(int device, int fp64, double *lane_ops_per_s);
 /* Diagnostics of the pruned KNN search (waits for the stream), both counted
  * since the previous call and then reset to 0:
- *   candidates_evaluated  candidates whose distance it computed (required)
- *   redo_pixels           pixels its walk could not finish and handed to the
- *                         redo pass (nullable): the disk of a pixel left the
- *                         staged tile, its undecided-key buffer overflowed,
- *                         the offset table held fewer than K valid offsets,
- *                         or nbr_idx was requested (then every pixel) */
+ *   candidates_evaluated  candidates whose distance decided something
+ *                         (required): the shell of the K-th offset for a
+ *                         pixel whose whole disk is taken without a search,
+ *                         every candidate of the disk for the others
+ *   redo_pixels           pixels left to the unbounded walk (nullable): more
+ *                         undecided keys than the buffer holds, candidates
+ *                         beyond the offset table, fewer than K valid offsets
+ *                         in it, or nbr_idx was requested (then every pixel) */
 hsc_status hsc_knn_diagnostics(hsc_ctx *ctx, int64_t *candidates_evaluated,
                                int64_t *redo_pixels);
 /* Testing aid for the device-side timeout path (no counterpart in the

@@ -1029,7 +1029,8 @@ bool staged_batch_ok(const hsc_frame *frames, int n_frames, int B, const hsc_knn
     for (int f = 0; f < n_frames; ++f) {
         const long N = (long)frames[f].H * frames[f].W;
         if (!hsc::gram_tc_usable(frames[f].cube, B, N)) return false;
-        ctas += (long)frames[f].H * ((frames[f].W + 31) / 32);
+        // the KNN grid's CTAs and the fused kernel's row segments both fit an int
+        ctas += (long)frames[f].H * ((frames[f].W + 31) / 32) + N / 32 + 2;
     }
     return ctas < (1L << 31);
 }
@@ -1059,7 +1060,7 @@ hsc_status classify_batch_staged(hsc_ctx *ctx, const hsc_frame *frames, int n_fr
         off = align_up(off + bytes);
         return o;
     };
-    int n_gram = 0, n_pix = 0, n_ctas = 0, max_rows = 1;
+    int n_gram = 0, n_pix = 0, n_ctas = 0, n_seg = 0, max_rows = 1;
     for (int f = 0; f < n_frames; ++f) {
         const hsc_frame &fr = frames[f];
         const long N = (long)fr.H * fr.W;
@@ -1085,7 +1086,8 @@ hsc_status classify_batch_staged(hsc_ctx *ctx, const hsc_frame *frames, int n_fr
         L.Iraw = take(sizeof(float) * (size_t)N);
         n_gram += L.parts;
         n_pix += (int)((N + kPixPerItem - 1) / kPixPerItem);
-        n_ctas += fr.H * ((fr.W + 31) / 32);
+        n_ctas += hsc::batch_knn_ctas(fr.H, fr.W, params->k, R);
+        n_seg += fr.H * ((fr.W + 31) / 32);
         max_rows = std::max(max_rows, std::min(R, fr.H));
     }
     long n_px = 0;
@@ -1168,9 +1170,9 @@ hsc_status classify_batch_staged(hsc_ctx *ctx, const hsc_frame *frames, int n_fr
     int *hc = reinterpret_cast<int *>(host + align_up(tab_frames) + tab_gram + tab_pix + tab_large);
     // frame groups: the first sm frames (one wave of Jacobi CTAs) and the rest
     const int F1 = n_frames > sm ? sm : n_frames;
-    int ip_split = 0, cta_split = 0;
+    int ip_split = 0, cta_split = 0, seg_split = 0;
     long px_split = 0;
-    int ig = 0, ip = 0, cta = 0, il = 0;
+    int ig = 0, ip = 0, cta = 0, seg = 0, il = 0;
     for (int f = 0; f < n_frames; ++f) {
         const hsc_frame &fr = frames[f];
         const FrameLay &L = fl[(size_t)f];
@@ -1178,6 +1180,7 @@ hsc_status classify_batch_staged(hsc_ctx *ctx, const hsc_frame *frames, int n_fr
         if (f == F1) {
             ip_split = ip;
             cta_split = cta;
+            seg_split = seg;
         }
         if (f < F1) px_split += N;
         BatchFrame b{};
@@ -1205,6 +1208,7 @@ hsc_status classify_batch_staged(hsc_ctx *ctx, const hsc_frame *frames, int n_fr
         b.per = (int)L.per;
         b.vec = L.vec;
         b.knn_cta0 = cta;
+        b.knn_seg0 = seg;
         b.Iraw = reinterpret_cast<float *>(dev + L.Iraw);
         b.svm_items = 0;
         const long total_chunks = (N + 63) / 64;
@@ -1229,7 +1233,8 @@ hsc_status classify_batch_staged(hsc_ctx *ctx, const hsc_frame *frames, int n_fr
             ++b.svm_items;
         }
         hf[f] = b;
-        cta += fr.H * ((fr.W + 31) / 32);
+        cta += hsc::batch_knn_ctas(fr.H, fr.W, params->k, R);
+        seg += fr.H * ((fr.W + 31) / 32);
         if (N > 4096) hl[il++] = f;
     }
     {
@@ -1286,7 +1291,7 @@ hsc_status classify_batch_staged(hsc_ctx *ctx, const hsc_frame *frames, int n_fr
         int lam_bits;
         memcpy(&lam_bits, &params->lambda, sizeof lam_bits);
         sig = {n_frames, B, (long long)flags, k, params->k, R, lam_bits, n_gram, n_pix, n_ctas,
-               max_rows, n_large, F1, ip_split, cta_split, (long long)px_split,
+               n_seg, max_rows, n_large, F1, ip_split, cta_split, seg_split, (long long)px_split,
                reinterpret_cast<long long>(model->w), reinterpret_cast<long long>(model->b),
                reinterpret_cast<long long>(model->platt_a),
                reinterpret_cast<long long>(model->platt_b),
@@ -1307,8 +1312,8 @@ hsc_status classify_batch_staged(hsc_ctx *ctx, const hsc_frame *frames, int n_fr
     // the stages after the moments for frames [f0, f1) of the table: the
     // eigensolvers, then projection/SVM, normalisation and KNN over the
     // group's work items, CTAs and redo-list share
-    auto tail = [&](int f0, int f1, int ip0, int ip1, int cta0, int cta1, long px0, long px1,
-                    cudaStream_t s, bool with_jacobi) -> cudaError_t {
+    auto tail = [&](int f0, int f1, int ip0, int ip1, int cta0, int cta1, int seg0, int seg1,
+                    long px0, long px1, cudaStream_t s, bool with_jacobi) -> cudaError_t {
         cudaError_t r = cudaSuccess;
         if (with_jacobi) {
             StageTimer t(tc, HSC_STAGE_JACOBI, 2, s);  // the lean form and the guarded full one
@@ -1319,8 +1324,8 @@ hsc_status classify_batch_staged(hsc_ctx *ctx, const hsc_frame *frames, int n_fr
             // (+ the redo pass); its time is booked to the KNN stage
             StageTimer t(tc, HSC_STAGE_KNN, 2, s);
             unsigned *claim = reinterpret_cast<unsigned *>(dev + claims) + (f0 == 0 ? 0 : 2);
-            r = hsc::launch_batch_svm_knn(df, dp + ip0, ip1 - ip0, df + f0, f1 - f0, cta1 - cta0,
-                                          cta0, B, model, f64, params->k, R, params->lambda,
+            r = hsc::launch_batch_svm_knn(df, dp + ip0, ip1 - ip0, df + f0, f1 - f0, seg1 - seg0,
+                                          seg0, B, model, f64, params->k, R, params->lambda,
                                           !(flags & HSC_CLASSIFY_RAW_I), max_rows,
                                           redo_list + px0, (unsigned)(px1 - px0), claim, sm, s);
             return r;
@@ -1336,8 +1341,8 @@ hsc_status classify_batch_staged(hsc_ctx *ctx, const hsc_frame *frames, int n_fr
         if (r == cudaSuccess) {
             StageTimer t(tc, HSC_STAGE_KNN, 2, s);
             r = hsc::launch_batch_knn(df + f0, f1 - f0, cta1 - cta0, cta0, k, params->k, R,
-                                      params->lambda, max_rows, redo_list + px0,
-                                      (unsigned)(px1 - px0), s);
+                                      params->lambda, redo_list + px0, (unsigned)(px1 - px0),
+                                      s);
         }
         return r;
     };
@@ -1346,7 +1351,7 @@ hsc_status classify_batch_staged(hsc_ctx *ctx, const hsc_frame *frames, int n_fr
         e = hsc::launch_batch_moments(df, n_frames, dg, dc, n_gram, dl, n_large, B, sm, st);
     }
     if (e == cudaSuccess && F1 == n_frames) {
-        e = tail(0, n_frames, 0, n_pix, 0, n_ctas, 0, n_px, st, true);
+        e = tail(0, n_frames, 0, n_pix, 0, n_ctas, 0, n_seg, 0, n_px, st, true);
     } else if (e == cudaSuccess) {
         // more frames than SMs: the eigensolvers take two waves. The second
         // group's chain runs on a high-priority stream (its Jacobi CTAs take
@@ -1369,10 +1374,12 @@ hsc_status classify_batch_staged(hsc_ctx *ctx, const hsc_frame *frames, int n_fr
         }
         if (e == cudaSuccess) e = cudaEventRecord(ctx->sm_ev[1], hi);
         if (e == cudaSuccess)
-            e = tail(F1, n_frames, ip_split, n_pix, cta_split, n_ctas, px_split, n_px, hi, true);
+            e = tail(F1, n_frames, ip_split, n_pix, cta_split, n_ctas, seg_split, n_seg, px_split,
+                     n_px, hi, true);
         if (e == cudaSuccess) e = cudaEventRecord(ctx->sm_ev[2], hi);
         if (e == cudaSuccess) e = cudaStreamWaitEvent(st, ctx->sm_ev[1], 0);
-        if (e == cudaSuccess) e = tail(0, F1, 0, ip_split, 0, cta_split, 0, px_split, st, false);
+        if (e == cudaSuccess)
+            e = tail(0, F1, 0, ip_split, 0, cta_split, 0, seg_split, 0, px_split, st, false);
         if (e == cudaSuccess) e = cudaStreamWaitEvent(st, ctx->sm_ev[2], 0);
     }
     if (graph) {

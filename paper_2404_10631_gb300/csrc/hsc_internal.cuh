@@ -121,7 +121,8 @@ struct BatchFrame {
     int n_part;          // partial Grams (tensor-core items of the frame)
     int per;             // 64-pixel chunks per partial
     int vec;             // 16-byte loads: cube 16-byte aligned and N % 4 == 0
-    int knn_cta0;        // first CTA of the frame in the batched KNN grid
+    int knn_cta0;        // first CTA of the frame in the batched KNN grid (tiled walk)
+    int knn_seg0;        // first 32-pixel row segment of the frame in the fused kernel's KNN
     float *Iraw;         // N: the raw projection (the fused kernel normalises into I)
     int svm_items;       // projection/SVM work items of the frame
 };
@@ -155,19 +156,13 @@ struct Tuning {
     int gram_stages = 0;
     int svm_px = 0;
     int svm_blocks_per_sm = 0;
-    int knn_variant = 4;  // launch_knn's variant of the pruned walk (4: 32 x 8, TMA tile)
+    int knn_variant = 4;  // launch_knn's variant of the pruned walk (4 warps per CTA)
 };
 
 cudaError_t launch_moments(const float *cube, int B, long N, const PcaScratch &s,
                            int sm_count, cudaStream_t st, bool force_simt = false,
                            int gram_stages = 0);
 bool gram_tc_supported(const float *cube, int B, long N);  // through a tensor map
-// A 2-D tensor map of a rows x cols float32 array (row-major, no swizzle,
-// out-of-range boxes read as zero) with box_cols x box_rows boxes; false when
-// the array or the box breaks a tensor-map rule (cols * 4 and box_cols * 4
-// multiples of 16 bytes, a 16-byte-aligned base) or the driver lacks the call.
-bool encode_map_2d_f32(CUtensorMap *map, const float *base, long rows, long cols, int box_cols,
-                       int box_rows);
 bool gram_tc_usable(const float *cube, int B, long N);     // tensor map or work items
 int moments_kernel_count(const float *cube, int B, long N, bool force_simt = false);
 cudaError_t launch_gram_tc(const float *cube, int B, long N, const PcaScratch &s,
@@ -199,8 +194,10 @@ cudaError_t launch_batch_project_svm(const BatchFrame *frames, const PixItem *it
 cudaError_t launch_batch_normalize(const BatchFrame *frames, const PixItem *items, int n_items,
                                    cudaStream_t st);
 cudaError_t launch_batch_knn(const BatchFrame *frames, int n_frames, int n_ctas, int cta_base,
-                             int k, int K, int R, float lambda, int max_rows, int2 *redo_list,
+                             int k, int K, int R, float lambda, int2 *redo_list,
                              unsigned redo_cap, cudaStream_t st);
+// CTAs of one frame in that grid.
+int batch_knn_ctas(int H, int W, int K, int R);
 // The projection/SVM, normalisation and KNN of a group of frames in one
 // persistent launch (work items first, then the KNN row segments, which wait
 // for their frame's items), then the redo pass; normalize false leaves I raw
@@ -258,12 +255,10 @@ cudaError_t launch_bip_to_bsq(const float *bip, int B, long N, float *bsq, cudaS
 cudaError_t knn_init(int device);
 
 // P4 (nullable): P pixel-interleaved, (k + 3) / 4 float4 per pixel, which
-// the pruned search gathers from (one 16-byte load per 4 classes).
-// variant (pruned search with P4): the walk's pixels per CTA and undecided
-// keys per lane, 0 = 32 and 8, 1 = 32 and 6, 2 = 32 and 12, 3 = 64 and 8,
-// 4 = 32 and 8 and 5 = 64 and 8 with the window tile staged by one TMA box
-// (where the map allows a tensor map; else as 0 and 3); the outputs do not
-// depend on it.
+// the pruned search reads (one 16-byte load per 4 classes).
+// variant (pruned search): the warps per CTA of the tiled walk, 0 = 4,
+// 1 = 1, 2 = 2, 3 = 8, 4 = 4 (the default), 5 = 6; the outputs do not depend
+// on it.
 constexpr int kKnnVariants = 6;
 cudaError_t launch_knn(const float *I, const float *P, int k, int H, int W, int K, int R,
                        float lambda, float *O, int32_t *labels, int32_t *nbr,

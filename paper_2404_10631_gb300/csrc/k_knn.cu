@@ -25,7 +25,6 @@
 #include <cuda_runtime.h>
 
 #include <atomic>
-#include <cstring>
 #include <math.h>
 
 #include <algorithm>
@@ -34,8 +33,8 @@
 #include <vector>
 
 #include "hsc_internal.cuh"
+#include "knn_generic.cuh"
 #include "svm_pixel.cuh"
-#include "tma_util.cuh"
 
 namespace hsc {
 namespace {
@@ -47,45 +46,9 @@ constexpr int kStride = kChunk + 4;         // shared row stride (floats)
 constexpr int kCap = HSC_MAX_K + 32;        // per-lane candidate buffer
 constexpr float kMargin = 1.0f / 262144.f;  // 2^-18 relative filter slack
 
-// Offsets (dr, dc) with dr^2 + dc^2 <= 400 and |dr| <= 16, sorted by
-// s = dr^2 + dc^2 (then dr, dc), built on the host once per device.
-constexpr int kTabR2 = 400;            // table: dr^2 + dc^2 <= 400
-constexpr int kTabDr = 16;             // |dr| <= 16: windows of up to 32 rows
-constexpr int kTabDc = 20;             // |dc| <= 20 follows from kTabR2
-constexpr int kTabCap = 1200;
-__constant__ char2 c_knn_tab[kTabCap];
-__constant__ int c_knn_tab_n;
 // extent of the first K table offsets (K = 1..64): max |dr| above and below,
 // max |dc|, and s of the K-th
 __constant__ char4 c_knn_pref[HSC_MAX_K + 1];
-
-struct Key {
-    float hi, lo;
-    int q;
-};
-
-__device__ __forceinline__ bool key_le(const Key &a, const Key &b)
-{
-    return a.hi < b.hi || (a.hi == b.hi && (a.lo < b.lo || (a.lo == b.lo && a.q <= b.q)));
-}
-__device__ __forceinline__ bool key_lt(const Key &a, const Key &b)
-{
-    return a.hi < b.hi || (a.hi == b.hi && (a.lo < b.lo || (a.lo == b.lo && a.q < b.q)));
-}
-
-// Exact distance as (hi, lo) = s + e (Knuth's TwoSum, round-to-nearest ops).
-__device__ __forceinline__ Key make_key(float Ip, float Iq, int dr, int dc, float l2, int q)
-{
-    float dI = __fsub_rn(Ip, Iq);
-    float e = __fmul_rn(dI, dI);
-    float s = __fmul_rn(l2, (float)(dr * dr + dc * dc));
-    Key k;
-    k.hi = __fadd_rn(s, e);
-    float bb = __fsub_rn(k.hi, s);
-    k.lo = __fadd_rn(__fsub_rn(s, __fsub_rn(k.hi, bb)), __fsub_rn(e, bb));
-    k.q = q;
-    return k;
-}
 
 // Per-row filter threshold for the current bound tau: a candidate of row
 // offset dr can only have key <= tau if fma(dI, dI, lambda^2 dc^2) <= this.
@@ -139,11 +102,6 @@ __device__ float canonical_L(int r, int c, int lo_r, int hi_r, int W, int K, flo
     }
     sK = 0;
     return -INFINITY;
-}
-
-__device__ __forceinline__ bool below_L(const Key &a, float L)
-{
-    return a.hi < L || (a.hi == L && a.lo < 0.f);
 }
 
 // Writes the pixel's outputs from its K selected keys: neighbour indices
@@ -453,7 +411,9 @@ knn_heap_kernel(const float *__restrict__ I, const float *__restrict__ P, int k,
                  W, l2);
 }
 
-// ---- exact, spatially pruned variant (lambda > 0)
+// ---- exact, spatially pruned variant (lambda > 0): the walk of the batch's
+// fused kernel (a warp per 32 pixels of a row; the other forms take the tiled
+// walk, knn_tile_kernel.cuh, on the same bounds) and the redo pass
 //
 // Every key is at least s_term = fl(lambda^2 (dr^2 + dc^2)), which grows with
 // the squared spatial distance s = dr^2 + dc^2. Let s_K be the K-th smallest
@@ -462,7 +422,7 @@ knn_heap_kernel(const float *__restrict__ I, const float *__restrict__ P, int k,
 // lies in [L, tau] for any upper bound tau. Then:
 //  * tau: for a pixel whose K spatially nearest offsets (the first K of a
 //    table of offsets sorted by s) all lie in the window, tau = L + e_max,
-//    rounded up, with e_max = (max I - min I)^2 over the CTA's I tile; near
+//    rounded up, with e_max = (max I - min I)^2 over the warp's I tile; near
 //    the image edges, the largest key of the first K valid offsets of the
 //    table (a walk with validity checks);
 //  * the disk s_term <= tau is walked row by row from the I tile staged in
@@ -475,11 +435,11 @@ knn_heap_kernel(const float *__restrict__ I, const float *__restrict__ P, int k,
 //    kind) complete the set: the same set as the full-window scan.
 // A pixel that cannot finish this way (its disk leaves the tile, the buffer
 // cannot hold the undecided keys, fewer than K valid offsets in the table,
-// or neighbour-index output) gets the sentinel label kRedoLabel and
-// knn_redo_kernel completes it with an unbounded walk.
+// or neighbour-index output) gets the sentinel label kRedoLabel; the second
+// pass tries box_pixel with a larger buffer (not for neighbour-index output),
+// then completes it with an unbounded walk.
 constexpr int kWalkThreads = 32;
 constexpr int kBnd = 8;                // undecided keys per lane
-constexpr int kRedoLabel = -2147483647 - 1;
 constexpr int kBatchRedoCtas = 1024;  // the batched redo pass's grid (exits at once when idle)
 constexpr int kRedoThreads = 32;
 constexpr int kRedoExtra = 32;         // redo buffer slots beyond K
@@ -586,72 +546,27 @@ __device__ __forceinline__ void add_probs4_coherent(float (&acc)[KC], const floa
     }
 }
 
-template <int KC, bool kP4, bool kCoherent = false>
-__device__ __forceinline__ void gather_probs(float (&acc)[KC], const float *__restrict__ P, long N,
-                                             const float4 *__restrict__ P4, int q)
-{
-    if (kCoherent) add_probs4_coherent(acc, P4, q);
-    else if (kP4) add_probs4(acc, P4, q);
-    else add_probs(acc, P, N, q);
-}
-
+// The pruned walk of one row segment by one warp (the batch's fused
+// projection/SVM + KNN kernel; the other forms take the tiled walk,
+// knn_tile_kernel.cuh): 32 pixels of row r from column bx * 32, a lane per
+// pixel, the window rows staged in sm (the tile, then the lanes'
+// undecided-key buffers). norm: the tile is read from the raw projection I
+// and normalised in shared memory with the frame's minimum nmin and range
+// nrange, the same expression as the normalisation pass, and each lane writes
+// its own pixel's normalised value to I_out. The probabilities are read with
+// plain loads (they are written earlier in the same launch). frames, frame:
+// the batch's table and this segment's index in it (redo list).
 template <int KC>
-__device__ __forceinline__ void write_pixel(const float (&acc)[KC], int K, long N, long p,
-                                            float *__restrict__ O, int32_t *__restrict__ labels)
-{
-    const float invK = 1.f / (float)K;
-    int best = 0;
-    float bestv = -INFINITY;
-#pragma unroll
-    for (int cl = 0; cl < KC; ++cl) {
-        const float o = acc[cl] * invK;
-        if (O) O[(size_t)cl * (size_t)N + p] = o;
-        if (o > bestv) {
-            bestv = o;
-            best = cl;
-        }
-    }
-    labels[p] = best;
-}
-
-// The pruned walk of one row segment: kWT pixels of row r from column
-// bx * kWT, a lane per pixel (lane in 0 .. kWT-1), the window rows staged in
-// sm (the tile, then the lanes' undecided-key buffers). kWarp: the segment is
-// one warp of a larger CTA (kWT == 32; warp-level synchronisation, no shared
-// reduction). norm: the tile is read from the raw projection I and
-// normalised in shared memory with the frame's minimum nmin and range
-// nrange, the same expression as the normalisation pass, and each lane
-// writes its own pixel's normalised value to I_out. kCoherent: plain loads
-// of the probabilities (written earlier in the same launch). frames, frame:
-// a stage-major batch's table and this segment's index in it (redo list).
-template <int KC, bool kBatch, bool kP4, int kWT, int kBN, bool kWarp = false,
-          bool kCoherent = false>
-__device__ __forceinline__ void knn_walk(const float *__restrict__ I, const float *__restrict__ P,
-                                         int H, int W, int K, int R, float lam,
-                                         float *__restrict__ O, int32_t *__restrict__ labels,
-                                         bool redo_all, Control *ctl,
+__device__ __forceinline__ void knn_walk(const float *__restrict__ I, int H, int W, int K, int R,
+                                         float lam, float *__restrict__ O,
+                                         int32_t *__restrict__ labels, Control *ctl,
                                          const BatchFrame *__restrict__ frames, int frame,
                                          int2 *__restrict__ redo_list, unsigned redo_cap,
                                          const float4 *P4, int r, int bx, int lane, float *sm,
-                                         float *s_min, float *s_max, bool norm = false,
-                                         float nmin = 0.f, float nrange = 0.f,
-                                         float *__restrict__ I_out = nullptr,
-                                         const CUtensorMap *tmap = nullptr,
-                                         uint64_t *tbar = nullptr)
+                                         bool norm, float nmin, float nrange,
+                                         float *__restrict__ I_out)
 {
-    static_assert(!kWarp || kWT == 32, "a warp-scope segment is one warp");
-    auto sync = [] {
-        if constexpr (kWarp) __syncwarp();
-        else __syncthreads();
-    };
-    auto any = [](bool v) -> bool {
-        if constexpr (kWarp) return __any_sync(0xffffffffu, v) != 0;
-        else return __syncthreads_or(v) != 0;
-    };
-    auto count = [](bool v) -> unsigned {
-        if constexpr (kWarp) return (unsigned)__popc(__ballot_sync(0xffffffffu, v));
-        else return (unsigned)__syncthreads_count(v);
-    };
+    constexpr int kWT = kWalkThreads, kBN = kBnd;
     auto nrm = [&](float v) { return (nrange > 0.f) ? (v - nmin) / nrange : 0.f; };
     const int c0 = bx * kWT, c = c0 + lane;
     const bool active = c < W;
@@ -659,10 +574,7 @@ __device__ __forceinline__ void knn_walk(const float *__restrict__ I, const floa
     const int hi_r = min(H - 1, r + (R + 1) / 2 - 1);
     const int nrows = hi_r - lo_r + 1;
     const int tw = kWT + 2 * kTabDc, tcol0 = c0 - kTabDc;
-    // nrows x tw (with a tensor map: 128-byte aligned, the launch adds 128 bytes)
-    float *tile = tmap ? reinterpret_cast<float *>((reinterpret_cast<uintptr_t>(sm) + 127) &
-                                                   ~static_cast<uintptr_t>(127))
-                       : sm;
+    float *tile = sm;  // nrows x tw
     LaneBuf bnd;
     bnd.stride = kWT;
     bnd.hi = tile + nrows * tw + lane;
@@ -679,32 +591,7 @@ __device__ __forceinline__ void knn_walk(const float *__restrict__ I, const floa
     static_assert((kWT + 2 * kTabDc) % 4 == 0 && kTabDc % 4 == 0, "tile rows of float4");
     const bool vec = tcol0 >= 0 && tcol0 + tw <= W && (W & 3) == 0 &&
                      (reinterpret_cast<uintptr_t>(I) & 15u) == 0;
-    if (tmap) {
-        // one box of the map's tensor map: rows lo_r .. lo_r + box rows - 1,
-        // columns tcol0 .. tcol0 + tw - 1 (tcol0 * 4 bytes is a multiple of
-        // 16: c0 is a multiple of 32 and kTabDc of 4); entries outside the
-        // map read as zero, as the 4-byte copies below zero-fill them
-        static_assert(kTabDc % 4 == 0 && kWT % 4 == 0, "a 16-byte-aligned box start");
-        if (lane == 0) {
-            tma::mbar_init(tbar, 1);
-            asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-        }
-        sync();
-        if (lane == 0) {
-            const int box_rows = R < H ? R : H;
-            tma::mbar_arrive_tx(tbar, (uint32_t)(box_rows * tw * (int)sizeof(float)));
-            tma::tma_load_2d(tile, tmap, tcol0, lo_r, tbar);
-        }
-        volatile int gave_up = 0;
-        const bool landed = tma::mbar_wait(tbar, 0, &gave_up);
-        bool all_landed;
-        if constexpr (kWarp) all_landed = __all_sync(0xffffffffu, landed) != 0;
-        else all_landed = __syncthreads_and(landed) != 0;
-        if (!all_landed) {  // the copy did not arrive within the bound: report and stop
-            if (lane == 0) atomicOr(&ctl->status, ST_TIMEOUT);
-            return;
-        }
-    } else if (vec) {
+    if (vec) {
         for (int idx = lane; idx < nrows * kV; idx += kWT) {
             const int ii = idx / kV, v = idx - ii * kV;
             const unsigned dst = (unsigned)__cvta_generic_to_shared(tile + ii * tw + 4 * v);
@@ -725,10 +612,8 @@ __device__ __forceinline__ void knn_walk(const float *__restrict__ I, const floa
             }
         }
     }
-    if (!tmap) {
-        asm volatile("cp.async.wait_all;" ::: "memory");
-        sync();
-    }
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    __syncwarp();
     bool bad = false;
     float vmin = INFINITY, vmax = -INFINITY;
     if (vec) {
@@ -757,26 +642,12 @@ __device__ __forceinline__ void knn_walk(const float *__restrict__ I, const floa
         vmin = fminf(vmin, __shfl_xor_sync(0xffffffffu, vmin, o));
         vmax = fmaxf(vmax, __shfl_xor_sync(0xffffffffu, vmax, o));
     }
-    if constexpr (kWarp) {
-        __syncwarp();  // the normalised tile before any lane reads it
-    } else {
-        if ((lane & 31) == 0) {
-            s_min[lane >> 5] = vmin;
-            s_max[lane >> 5] = vmax;
-        }
-        __syncthreads();
-        vmin = s_min[0];
-        vmax = s_max[0];
-        for (int w = 1; w < kWT / 32; ++w) {
-            vmin = fminf(vmin, s_min[w]);
-            vmax = fmaxf(vmax, s_max[w]);
-        }
-    }
+    __syncwarp();  // the normalised tile before any lane reads it
 
     const float Ip = active ? tile[(r - lo_r) * tw + (c - tcol0)] : 0.f;
     if (norm && active) I_out[(long)r * W + c] = Ip;
     unsigned evals = 0;
-    bool redo = active && redo_all;
+    bool redo = false;
 
     // the bound tau and s_K
     const char4 pf = c_knn_pref[K];  // (max dr above, max dr below, max |dc|, s of the K-th)
@@ -844,7 +715,7 @@ __device__ __forceinline__ void knn_walk(const float *__restrict__ I, const floa
                 const float h = __fadd_rn(st, e);
                 if (h < L) {  // one of the K nearest
                     ++m;
-                    gather_probs<KC, kP4, kCoherent>(acc, P, N, P4, qrow + j);
+                    add_probs4_coherent(acc, P4, qrow + j);
                     continue;
                 }
                 if (h > tau.hi) continue;
@@ -853,7 +724,7 @@ __device__ __forceinline__ void knn_walk(const float *__restrict__ I, const floa
                 const Key kk = {h, lo, qrow + j};
                 if (h == L && lo < 0.f) {
                     ++m;
-                    gather_probs<KC, kP4, kCoherent>(acc, P, N, P4, qrow + j);
+                    add_probs4_coherent(acc, P4, qrow + j);
                     continue;
                 }
                 if (!key_le(kk, tau)) continue;
@@ -872,12 +743,7 @@ __device__ __forceinline__ void knn_walk(const float *__restrict__ I, const floa
         }
     }
     bad |= active && !isfinite(Ip);
-    if (any(bad) && lane == 0) atomicOr(&ctl->status, ST_NONFINITE_MAP);
-    const unsigned nredo = count(redo);
-    if (lane == 0 && nredo) {
-        if (!kBatch) atomicAdd(&ctl->knn_redo, nredo);
-        atomicAdd(&ctl->knn_redo_total, (unsigned long long)nredo);
-    }
+    if (__any_sync(0xffffffffu, bad) && lane == 0) atomicOr(&ctl->status, ST_NONFINITE_MAP);
     {
         unsigned long long e = evals;
         for (int o = 16; o > 0; o >>= 1) e += __shfl_xor_sync(0xffffffffu, e, o);
@@ -885,13 +751,11 @@ __device__ __forceinline__ void knn_walk(const float *__restrict__ I, const floa
     }
     if (!active) return;
     const long p = (long)r * W + c;
-    // a stage-major batch lists the pixels for its redo pass (frame, pixel)
+    // the batch lists the pixels for its redo pass (frame, pixel)
     auto to_redo = [&]() {
         labels[p] = kRedoLabel;
-        if (kBatch) {
-            const unsigned i = atomicAdd(&frames[0].ctl->knn_redo_list, 1u);
-            if (i < redo_cap) redo_list[i] = make_int2(frame, (int)p);
-        }
+        const unsigned i = atomicAdd(&frames[0].ctl->knn_redo_list, 1u);
+        if (i < redo_cap) redo_list[i] = make_int2(frame, (int)p);
     };
     if (redo) {
         to_redo();
@@ -900,8 +764,6 @@ __device__ __forceinline__ void knn_walk(const float *__restrict__ I, const floa
     const int need = K - m;
     if (need > nb) {  // cannot happen: the K-th smallest key is <= tau
         to_redo();
-        if (!kBatch) atomicAdd(&ctl->knn_redo, 1u);
-        atomicAdd(&ctl->knn_redo_total, 1ull);
         return;
     }
     // the need smallest undecided keys: need passes of a minimum search
@@ -919,57 +781,24 @@ __device__ __forceinline__ void knn_walk(const float *__restrict__ I, const floa
             }
         }
         if (im != a) bnd.put(im, bnd.get(a));
-        gather_probs<KC, kP4, kCoherent>(acc, P, N, P4, best.q);
+        add_probs4_coherent(acc, P4, best.q);
     }
     write_pixel(acc, K, N, p, O, labels);
 }
 
 
-// kWT: pixels per CTA (one row segment, a lane per pixel); kBN: undecided
-// keys per lane. Neither changes a result (the canonical summation order
-// makes O independent of which pixels the redo pass completes); an
-// autotuner picks them per frame shape.
-template <int KC, bool kBatch = false, bool kP4 = false, int kWT = kWalkThreads, int kBN = kBnd>
-__global__ void __launch_bounds__(kWT)
-knn_pruned_kernel(const float *__restrict__ I, const float *__restrict__ P, int H, int W, int K,
-                  int R, float lam, float *__restrict__ O, int32_t *__restrict__ labels,
-                  bool redo_all, Control *ctl, const BatchFrame *__restrict__ frames,
-                  int n_frames, int2 *__restrict__ redo_list, unsigned redo_cap,
-                  const float4 *__restrict__ P4, int cta_base,
-                  const __grid_constant__ CUtensorMap tmap, int use_tma)
+// Neighbour-index output: every pixel goes to the redo pass, which keeps its
+// K keys in order.
+__global__ void __launch_bounds__(256)
+knn_mark_kernel(int32_t *__restrict__ labels, long N, Control *ctl)
 {
-    extern __shared__ float sm[];
-    __shared__ float s_min[kWT / 32], s_max[kWT / 32];
-    __shared__ __align__(8) uint64_t tbar;
-    int r = blockIdx.y, bx = blockIdx.x;
-    int frame = 0;
-    if (kBatch) {  // a stage-major batch: the frame whose CTA range holds this CTA
-        const int cta = (int)blockIdx.x + cta_base;
-        int lo = 0, hi = n_frames - 1;
-        while (lo < hi) {
-            const int mid = (lo + hi + 1) >> 1;
-            if (frames[mid].knn_cta0 <= cta) lo = mid;
-            else hi = mid - 1;
-        }
-        frame = lo;
-        const BatchFrame &fr = frames[lo];
-        I = fr.I;
-        P = fr.P;
-        P4 = fr.P4;
-        H = fr.H;
-        W = fr.W;
-        O = fr.O;
-        labels = fr.labels;
-        ctl = fr.ctl;
-        const int t = cta - fr.knn_cta0;
-        const int tpr = (W + kWT - 1) / kWT;
-        r = t / tpr;
-        bx = t - r * tpr;
+    for (long p = (long)blockIdx.x * blockDim.x + threadIdx.x; p < N;
+         p += (long)gridDim.x * blockDim.x)
+        labels[p] = kRedoLabel;
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        ctl->knn_redo = (unsigned)N;  // N < 2^31
+        ctl->knn_redo_total += (unsigned long long)N;
     }
-    knn_walk<KC, kBatch, kP4, kWT, kBN>(I, P, H, W, K, R, lam, O, labels, redo_all, ctl, frames,
-                                        frame, redo_list, redo_cap, P4, r, bx, (int)threadIdx.x, sm,
-                                        s_min, s_max, false, 0.f, 0.f, nullptr,
-                                        use_tma ? &tmap : nullptr, &tbar);
 }
 
 template <int KC>
@@ -1124,11 +953,35 @@ __device__ __noinline__ void redo_pixel(const float *__restrict__ I, const float
 }
 
 
-// Completes the pixels knn_pruned_kernel left with the sentinel label: a walk
-// from global memory (the table in increasing s, then row by row over the
+constexpr int kRedoCap = 32;           // undecided keys per lane in box_pixel
+// box_pixel for the second pass, a warp together (todo: this lane has a
+// pixel): true where the pixel is left.
+template <int KC>
+__device__ __forceinline__ bool redo_box(const TileFrame &f, bool todo, long p, int K, int R,
+                                         float lam, float *sm)
+{
+    const Buf buf = {(uint32_t)__cvta_generic_to_shared(sm) + 4u * (threadIdx.x & 31)};
+    const float l2 = lam * lam;
+    const int q = todo ? (int)p : -1;
+    unsigned ev = f.P4 ? box_pixel<KC, true>(f, q, K, R, l2, buf, kRedoCap)
+                       : box_pixel<KC, false>(f, q, K, R, l2, buf, kRedoCap);
+    const bool left = ev == ~0u;
+    const unsigned n = __popc(__ballot_sync(0xffffffffu, left));
+    ev = __reduce_add_sync(0xffffffffu, left ? 0u : ev);
+    if ((threadIdx.x & 31) == 0) {
+        if (ev) atomicAdd(&f.ctl->knn_evals, (unsigned long long)ev);
+        if (n) atomicAdd(&f.ctl->knn_redo_total, (unsigned long long)n);  // the unbounded walk's
+    }
+    return left;
+}
+
+// Completes the pixels the pruned walk left with the sentinel label, 32
+// consecutive pixels per warp (left pixels come in clusters along the borders
+// of regions): box_pixel, and for what that leaves a walk from global memory
+// (the table in increasing s, then row by row over the
 // rest of the window, or of the disk s_term <= tau once K are in), keeping
 // every key <= tau in a buffer of K + 32 (compacted to the best K when full),
-// then the best K. A persistent grid; when the pruned kernel flagged nothing
+// then the best K. A persistent grid; when the walk flagged nothing
 // its CTAs exit at once, otherwise they scan the labels for the sentinel and
 // the last CTA to finish resets the counters.
 template <int KC>
@@ -1143,8 +996,14 @@ knn_redo_kernel(const float *__restrict__ I, const float *__restrict__ P, int H,
     for (long base = (long)blockIdx.x * kRedoThreads; base < N;
          base += (long)gridDim.x * kRedoThreads) {
         const long p = base + threadIdx.x;
-        if (p < N && labels[p] == kRedoLabel)
-            redo_pixel<KC>(I, P, H, W, K, R, lam, O, labels, nbr, ctl, p, sm, P4);
+        bool todo = p < N && labels[p] == kRedoLabel;
+        if (!__any_sync(0xffffffffu, todo)) continue;
+        if (!nbr) {
+            todo = redo_box<KC>({I, P, P4, O, labels, ctl, N, H, W}, todo, p, K, R, lam, sm);
+            __syncwarp();  // sm is shared with redo_pixel's buffers
+        }
+        if (todo) redo_pixel<KC>(I, P, H, W, K, R, lam, O, labels, nbr, ctl, p, sm, P4);
+        __syncwarp();
     }
     __syncthreads();
     if (threadIdx.x == 0) {
@@ -1170,12 +1029,18 @@ knn_redo_batch_kernel(const BatchFrame *__restrict__ frames, int K, int R, float
     unsigned n = *(volatile unsigned *)&c0->knn_redo_list;
     if (n > redo_cap) n = redo_cap;  // cannot happen: one entry per pixel at most
     if (n == 0u) return;
-    for (unsigned i = blockIdx.x * kRedoThreads + threadIdx.x; i < n;
-         i += gridDim.x * kRedoThreads) {
-        const int2 fp = redo_list[i];
+    for (unsigned i0 = blockIdx.x * kRedoThreads; i0 < n; i0 += gridDim.x * kRedoThreads) {
+        const unsigned i = i0 + threadIdx.x;
+        bool todo = i < n;
+        const int2 fp = redo_list[todo ? i : 0];
         const BatchFrame &fr = frames[fp.x];
-        redo_pixel<KC>(fr.I, fr.P, fr.H, fr.W, K, R, lam, fr.O, fr.labels, nullptr, fr.ctl,
-                       (long)fp.y, sm, fr.P4);
+        todo = redo_box<KC>({fr.I, fr.P, fr.P4, fr.O, fr.labels, fr.ctl, fr.N, fr.H, fr.W}, todo,
+                            (long)fp.y, K, R, lam, sm);  // (a frame per lane)
+        __syncwarp();
+        if (todo)
+            redo_pixel<KC>(fr.I, fr.P, fr.H, fr.W, K, R, lam, fr.O, fr.labels, nullptr, fr.ctl,
+                           (long)fp.y, sm, fr.P4);
+        __syncwarp();
     }
     __syncthreads();
     if (threadIdx.x == 0) {
@@ -1188,13 +1053,14 @@ knn_redo_batch_kernel(const BatchFrame *__restrict__ frames, int K, int R, float
     }
 }
 
-template <int kWT = kWalkThreads, int kBN = kBnd>
-size_t pruned_smem_bytes(int R, int H)
+// One warp's tile and undecided keys in the fused kernel.
+size_t walk_smem_bytes(int R, int H)
 {
     const int nrows = R < H ? R : H;
-    return sizeof(float) * ((size_t)nrows * (kWT + 2 * kTabDc) + 3 * (size_t)kBN * kWT);
+    return sizeof(float) * ((size_t)nrows * (kWalkThreads + 2 * kTabDc) + 3 * (size_t)kBnd * kWalkThreads);
 }
 
+static_assert(kRedoCap <= kRedoExtra, "box_pixel's buffer fits the redo pass's");
 size_t redo_smem_bytes(int K) { return sizeof(float) * 3 * (size_t)(K + kRedoExtra) * kRedoThreads; }
 
 // CTAs of the redo pass that the current device holds at once: SMs x the
@@ -1220,48 +1086,24 @@ long redo_resident_ctas(size_t smem)
     return n > 64 ? n : 64;
 }
 
-// tma: stage each CTA's window tile with one box of a tensor map of I, where
-// I allows one (W a multiple of 4 and at least the box width, a
-// 16-byte-aligned map); else 16- and 4-byte asynchronous copies.
-template <int KC, bool kP4, int kWT, int kBN>
-void launch_walk(const float *I, const float *P, int H, int W, int K, int R, float lam, float *O,
-                 int32_t *labels, int32_t *nbr, Control *ctl, cudaStream_t st, const float4 *P4,
-                 bool tma = false)
-{
-    CUtensorMap map;
-    memset(&map, 0, sizeof map);
-    const int rows = R < H ? R : H;
-    // (only where the box fits inside the map: narrower maps take the copies)
-    const bool use_tma =
-        tma && W >= kWT + 2 * kTabDc && encode_map_2d_f32(&map, I, H, W, kWT + 2 * kTabDc, rows);
-    const size_t smem = pruned_smem_bytes<kWT, kBN>(R, H) + (use_tma ? 128 : 0);
-    auto kern = knn_pruned_kernel<KC, false, kP4, kWT, kBN>;
-    if (smem > 48 * 1024)
-        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    dim3 grid((W + kWT - 1) / kWT, H);
-    kern<<<grid, kWT, smem, st>>>(I, P, H, W, K, R, lam, O, labels, nbr != nullptr, ctl, nullptr, 0,
-                                  nullptr, 0u, P4, 0, map, use_tma ? 1 : 0);
-}
+// Warps per CTA of the tiled walk by variant.
+constexpr int kTileWarps[kKnnVariants] = {4, 1, 2, 8, 4, 6};
+constexpr int kBatchTileWarps = 4;
 
-// variant (with the pixel-interleaved probabilities only): 0 = 32 pixels
-// per CTA and 8 undecided keys per lane (the default), 1 = 32 and 6,
-// 2 = 32 and 12, 3 = 64 and 8, 4 and 5 = 0 and 3 with the tile staged by TMA.
+// The tiled walk, then the redo pass over what it left.
 template <int KC>
 cudaError_t launch_pruned(const float *I, const float *P, int H, int W, int K, int R, float lam,
                           float *O, int32_t *labels, int32_t *nbr, Control *ctl, cudaStream_t st,
                           const float4 *P4, int variant = 0)
 {
-    if (P4) {
-        switch (variant) {
-        case 1: launch_walk<KC, true, 32, 6>(I, P, H, W, K, R, lam, O, labels, nbr, ctl, st, P4); break;
-        case 2: launch_walk<KC, true, 32, 12>(I, P, H, W, K, R, lam, O, labels, nbr, ctl, st, P4); break;
-        case 3: launch_walk<KC, true, 64, 8>(I, P, H, W, K, R, lam, O, labels, nbr, ctl, st, P4); break;
-        case 4: launch_walk<KC, true, 32, 8>(I, P, H, W, K, R, lam, O, labels, nbr, ctl, st, P4, true); break;
-        case 5: launch_walk<KC, true, 64, 8>(I, P, H, W, K, R, lam, O, labels, nbr, ctl, st, P4, true); break;
-        default: launch_walk<KC, true, 32, 8>(I, P, H, W, K, R, lam, O, labels, nbr, ctl, st, P4); break;
-        }
+    if (nbr) {
+        knn_mark_kernel<<<(unsigned)std::min<long>(((long)H * W + 255) / 256, 4096), 256, 0, st>>>(
+            labels, (long)H * W, ctl);
     } else {
-        launch_walk<KC, false, 32, 8>(I, P, H, W, K, R, lam, O, labels, nbr, ctl, st, nullptr);
+        const TileFrame f = {I, P, P4, O, labels, ctl, (long)H * W, H, W};
+        const cudaError_t e = launch_knn_tile(f, nullptr, 0, 0, 0, KC, K, R, lam, nullptr, 0u,
+                                              kTileWarps[variant], st);
+        if (e != cudaSuccess) return e;
     }
     const long N = (long)H * W;
     const size_t rsmem = redo_smem_bytes(K);
@@ -1280,18 +1122,13 @@ cudaError_t launch_pruned(const float *I, const float *P, int H, int W, int K, i
 
 template <int KC>
 cudaError_t launch_batch_pruned(const BatchFrame *frames, int n_frames, int n_ctas, int cta_base,
-                                int K, int R, float lam, int max_rows, int2 *redo_list,
-                                unsigned redo_cap, cudaStream_t st)
+                                int K, int R, float lam, int2 *redo_list, unsigned redo_cap,
+                                cudaStream_t st)
 {
-    const size_t smem = pruned_smem_bytes<>(R, max_rows);
-    if (smem > 48 * 1024)
-        cudaFuncSetAttribute(knn_pruned_kernel<KC, true, true>,
-                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    CUtensorMap none;
-    memset(&none, 0, sizeof none);
-    knn_pruned_kernel<KC, true, true><<<n_ctas, kWalkThreads, smem, st>>>(
-        nullptr, nullptr, 0, 0, K, R, lam, nullptr, nullptr, false, nullptr, frames, n_frames,
-        redo_list, redo_cap, nullptr, cta_base, none, 0);
+    const TileFrame none = {};
+    const cudaError_t e = launch_knn_tile(none, frames, n_frames, n_ctas, cta_base, KC, K, R, lam,
+                                          redo_list, redo_cap, kBatchTileWarps, st);
+    if (e != cudaSuccess) return e;
     const size_t rsmem = redo_smem_bytes(K);
     if (rsmem > 48 * 1024)
         cudaFuncSetAttribute(knn_redo_batch_kernel<KC>,
@@ -1397,12 +1234,12 @@ svm_knn_batch_kernel(const BatchFrame *__restrict__ frames, const PixItem *__res
         int lo = 0, hi = n_kframes - 1;
         while (lo < hi) {
             const int mid = (lo + hi + 1) >> 1;
-            if (kframes[mid].knn_cta0 <= cta) lo = mid;
+            if (kframes[mid].knn_seg0 <= cta) lo = mid;
             else hi = mid - 1;
         }
         const BatchFrame &fr = kframes[lo];
         const int tpr = (fr.W + 31) / 32;
-        const int t = cta - fr.knn_cta0;
+        const int t = cta - fr.knn_seg0;
         const int r = t / tpr, bx = t - r * tpr;
         int ok = 1;
         if (lane == 0) ok = wait_count(&fr.ctl->svm_done, (unsigned)fr.svm_items, fr.ctl) ? 1 : 0;
@@ -1419,10 +1256,9 @@ svm_knn_batch_kernel(const BatchFrame *__restrict__ frames, const PixItem *__res
             nmin = key_to_float(*(volatile const unsigned *)&fr.ctl->imin_key);
             nrange = key_to_float(*(volatile const unsigned *)&fr.ctl->imax_key) - nmin;
         }
-        knn_walk<KC, true, true, 32, kBnd, true, true>(
-            norm ? fr.Iraw : fr.I, fr.P, fr.H, fr.W, K, R, lam, fr.O, fr.labels, false, fr.ctl,
-            kframes, lo, redo_list, redo_cap, fr.P4, r, bx, lane, wsm, nullptr, nullptr,
-            norm != 0, nmin, nrange, fr.I);
+        knn_walk<KC>(norm ? fr.Iraw : fr.I, fr.H, fr.W, K, R, lam, fr.O, fr.labels, fr.ctl, kframes,
+                     lo, redo_list, redo_cap, fr.P4, r, bx, lane, wsm, norm != 0, nmin, nrange,
+                     fr.I);
         __syncwarp();
     }
 }
@@ -1436,7 +1272,7 @@ cudaError_t launch_batch_svm_knn_kc(const BatchFrame *frames, const PixItem *ite
                                     cudaStream_t st)
 {
     constexpr int M = KC * (KC - 1) / 2;
-    const int wfl = (int)(pruned_smem_bytes<32, kBnd>(R, max_rows) / sizeof(float));
+    const int wfl = (int)(walk_smem_bytes(R, max_rows) / sizeof(float));
     const size_t smem = sizeof(float) * std::max((size_t)B * (M + 2), (size_t)(kSvmThreads / 32) * wfl);
     auto kern = svm_knn_batch_kernel<KC>;
     if (smem > 48 * 1024)
@@ -1509,29 +1345,34 @@ cudaError_t knn_init(int device)
         side = std::max(side, std::abs(e[2]));
         pref[K] = make_char4((char)up, (char)down, (char)side, (char)e[0]);
     }
-    cudaError_t e = cudaMemcpyToSymbol(c_knn_tab, tab.data(), sizeof(char2) * tab.size());
-    if (e == cudaSuccess) e = cudaMemcpyToSymbol(c_knn_tab_n, &nt, sizeof(int));
+    cudaError_t e = upload_knn_tab(tab.data(), nt);
     if (e == cudaSuccess) e = cudaMemcpyToSymbol(c_knn_pref, pref.data(), sizeof(char4) * pref.size());
+    if (e == cudaSuccess) e = knn_tile_init(tab.data(), nt);
     if (e == cudaSuccess) done[device] = true;
     return e;
 }
 
-// Stage-major batch, pruned search (lambda > 0): n_ctas = sum over the
-// frames of H * ceil(W / 32), frame f's CTAs from frames[f].knn_cta0, the
-// first of them numbered cta_base; max_rows = the largest min(R, H).
+int batch_knn_ctas(int H, int W, int K, int R)
+{
+    return knn_tile_ctas(H, W, K, R, kBatchTileWarps);
+}
+
+// Stage-major batch, pruned search (lambda > 0): n_ctas = sum of
+// batch_knn_ctas over the frames, frame f's CTAs from frames[f].knn_cta0, the
+// first of them numbered cta_base.
 cudaError_t launch_batch_knn(const BatchFrame *frames, int n_frames, int n_ctas, int cta_base,
-                             int k, int K, int R, float lambda, int max_rows, int2 *redo_list,
+                             int k, int K, int R, float lambda, int2 *redo_list,
                              unsigned redo_cap, cudaStream_t st)
 {
     if (n_frames < 1 || n_ctas < 1 || !(lambda > 0.f) || !redo_list) return cudaErrorInvalidValue;
     switch (k) {
-    case 2: return launch_batch_pruned<2>(frames, n_frames, n_ctas, cta_base, K, R, lambda, max_rows, redo_list, redo_cap, st);
-    case 3: return launch_batch_pruned<3>(frames, n_frames, n_ctas, cta_base, K, R, lambda, max_rows, redo_list, redo_cap, st);
-    case 4: return launch_batch_pruned<4>(frames, n_frames, n_ctas, cta_base, K, R, lambda, max_rows, redo_list, redo_cap, st);
-    case 5: return launch_batch_pruned<5>(frames, n_frames, n_ctas, cta_base, K, R, lambda, max_rows, redo_list, redo_cap, st);
-    case 6: return launch_batch_pruned<6>(frames, n_frames, n_ctas, cta_base, K, R, lambda, max_rows, redo_list, redo_cap, st);
-    case 7: return launch_batch_pruned<7>(frames, n_frames, n_ctas, cta_base, K, R, lambda, max_rows, redo_list, redo_cap, st);
-    case 8: return launch_batch_pruned<8>(frames, n_frames, n_ctas, cta_base, K, R, lambda, max_rows, redo_list, redo_cap, st);
+    case 2: return launch_batch_pruned<2>(frames, n_frames, n_ctas, cta_base, K, R, lambda, redo_list, redo_cap, st);
+    case 3: return launch_batch_pruned<3>(frames, n_frames, n_ctas, cta_base, K, R, lambda, redo_list, redo_cap, st);
+    case 4: return launch_batch_pruned<4>(frames, n_frames, n_ctas, cta_base, K, R, lambda, redo_list, redo_cap, st);
+    case 5: return launch_batch_pruned<5>(frames, n_frames, n_ctas, cta_base, K, R, lambda, redo_list, redo_cap, st);
+    case 6: return launch_batch_pruned<6>(frames, n_frames, n_ctas, cta_base, K, R, lambda, redo_list, redo_cap, st);
+    case 7: return launch_batch_pruned<7>(frames, n_frames, n_ctas, cta_base, K, R, lambda, redo_list, redo_cap, st);
+    case 8: return launch_batch_pruned<8>(frames, n_frames, n_ctas, cta_base, K, R, lambda, redo_list, redo_cap, st);
     default: return cudaErrorInvalidValue;
     }
 }

@@ -32,8 +32,8 @@ def main(argv=None):
     ap.add_argument("--search", default="auto", choices=("auto", "full", "pruned", "heap"),
                     help="KNN search of --op knn")
     ap.add_argument("--knn-variant", type=int, default=None,
-                    help="pruned walk variant of --op classify (hsc_set_tuning; 4 and 5 stage "
-                         "the window tile by TMA); default: the untuned one")
+                    help="pruned walk variant of --op classify (hsc_set_tuning: warps per CTA); "
+                         "default: the untuned one")
     a = ap.parse_args(argv)
     sys.path.insert(0, os.path.dirname(os.path.abspath(__file__)))
     import torch
