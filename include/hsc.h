@@ -122,10 +122,10 @@ typedef struct {
 #define HSC_CUBE_BIP 32u
 /* flag for hsc_pca_one_band / hsc_classify: the eigensolver's plain form,
  * its basis from one Jacobi sweep on one CTA whatever the band count, where
- * by default B <= 128 takes two block power steps on C and 129 <= B <= 256 runs
- * the sweep on a thread-block cluster of 16 CTAs (8 where the device schedules
- * no clusters of 16). An A/B switch: every form reaches the same eigenpair to
- * the refinement's FP64-level tolerance. */
+ * by default up to 256 bands take a Krylov space of C (129 <= B <= 256 on a
+ * thread-block cluster of 8 CTAs), with the plain form behind it for frames
+ * that it does not separate. An A/B switch: every form reaches the same
+ * eigenpair to the refinement's FP64-level tolerance. */
 #define HSC_JACOBI_ONE_CTA 128u
 
 /* Create a context on `device`. cuda_stream: a cudaStream_t to launch on, or
@@ -355,7 +355,8 @@ enum {
 
 hsc_status hsc_profile_enable(hsc_ctx *ctx, int enable);
 /* Diagnostics of the context's last PCA (waits for the stream): FP32 Jacobi
- * sweeps run, FP64 refinement iterations of the leading eigenvector, and the
+ * sweeps run (the Krylov basis of 129-256 bands counts as one, that of up to
+ * 128 as none), FP64 refinement iterations of the leading eigenvector, and the
  * SM clock cycles spent in each part (cycle pointers nullable). */
 hsc_status hsc_pca_diagnostics(hsc_ctx *ctx, int32_t *sweeps, int32_t *refine_iters,
                                int64_t *sweep_cycles, int64_t *refine_cycles);

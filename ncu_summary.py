@@ -28,14 +28,14 @@ STAGE_OF = (("pilot_", "moments"), ("gram_tc_kernel", "moments"),
             ("gram_tc_items_kernel", "moments"), ("gram_tc_wide_kernel", "moments"),
             ("gram_partial_kernel", "moments"),
             ("gram_reduce_kernel", "moments"), ("jacobi_kernel", "jacobi"),
-            ("jacobi_cluster_kernel", "jacobi"),
+            ("jacobi_cluster_kernel", "jacobi"), ("krylov_kernel", "jacobi"),
             ("project_svm_kernel", "project_svm"), ("project_svm_batch_kernel", "project_svm"),
             ("normalize_kernel", "normalize"), ("normalize_batch_kernel", "normalize"),
             ("knn_tile_kernel", "knn"), ("knn_redo_kernel", "knn"),
             ("svm_knn_batch_kernel", "knn"),
             ("knn_redo_batch_kernel", "knn"), ("knn_kernel", "knn_full"))
 SOURCE_OF = {"moments": ("k_moments.cu", "k_gram_tc.cu", "dfloat.cuh"),
-             "jacobi": ("k_jacobi.cu", "k_jacobi_cluster.cu", "jacobi_rot.cuh", "dfloat.cuh"),
+             "jacobi": ("k_krylov.cu", "k_jacobi.cu", "k_jacobi_cluster.cu", "jacobi_rot.cuh", "dfloat.cuh"),
              "project_svm": ("k_project_svm.cu", "svm_pixel.cuh"),
              "normalize": ("k_project_svm.cu", "svm_pixel.cuh"),
              "knn": ("k_knn.cu", "knn_tile_kernel.cuh", "knn_generic.cuh", "knn_key.cuh", "svm_pixel.cuh"), "knn_full": ("k_knn.cu", "svm_pixel.cuh")}

@@ -196,7 +196,7 @@ Layout make_layout(const hsc_ctx *ctx, int B, long N, int k, bool need_pca, bool
         L.v1f = take(sizeof(float) * B);
         L.muf = take(sizeof(float) * B);
         L.jA = take(sizeof(float) * hsc::jacobi_global_floats(B));
-        if (hsc::jacobi_cluster_floats(B))  // the cluster sweep's V and diagonal
+        if (n_pc > 1 && hsc::jacobi_cluster_floats(B))  // the cluster sweep's V and diagonal
             L.jV = take(sizeof(float) * hsc::jacobi_cluster_floats(B));
         if (k > 0)  // the whole path: P pixel-interleaved for the KNN's gathers
             L.p4 = take(sizeof(float4) * (size_t)((k + 3) / 4) * (size_t)N);
@@ -1316,7 +1316,7 @@ hsc_status classify_batch_staged(hsc_ctx *ctx, const hsc_frame *frames, int n_fr
                     long px0, long px1, cudaStream_t s, bool with_jacobi) -> cudaError_t {
         cudaError_t r = cudaSuccess;
         if (with_jacobi) {
-            StageTimer t(tc, HSC_STAGE_JACOBI, 2, s);  // the lean form and the guarded full one
+            StageTimer t(tc, HSC_STAGE_JACOBI, 2, s);  // the Krylov form and the guarded full one
             r = hsc::launch_batch_jacobi(df + f0, f1 - f0, B, s);
         }
         if (r == cudaSuccess && (flags & HSC_BATCH_FUSED)) {
@@ -1369,7 +1369,7 @@ hsc_status classify_batch_staged(hsc_ctx *ctx, const hsc_frame *frames, int n_fr
         if (e == cudaSuccess) e = cudaEventRecord(ctx->sm_ev[0], st);
         if (e == cudaSuccess) e = cudaStreamWaitEvent(hi, ctx->sm_ev[0], 0);
         if (e == cudaSuccess) {
-            StageTimer t(tc, HSC_STAGE_JACOBI, 2, hi);  // the lean form and the guarded full one
+            StageTimer t(tc, HSC_STAGE_JACOBI, 2, hi);  // the Krylov form and the guarded full one
             e = hsc::launch_batch_jacobi(df, F1, B, hi);
         }
         if (e == cudaSuccess) e = cudaEventRecord(ctx->sm_ev[1], hi);

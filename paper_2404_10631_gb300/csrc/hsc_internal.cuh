@@ -49,7 +49,7 @@ struct Control {
                               // its first wait after a short bound (set and cleared by the host)
     unsigned long long knn_redo_total;  // pixels the pruned KNN left to its redo pass since last read
     unsigned long long jacobi_cluster_cycles;  // SM clock cycles of the cluster sweep (its CTA 0)
-    unsigned jac_redo;        // the lean eigensolver left this frame to the full one (reset by it)
+    unsigned jac_redo;        // the Krylov eigensolver left this frame to the full one (reset by it)
     unsigned svm_done;        // stage-major batch: projection/SVM items of the frame finished in
                               // the fused projection/SVM + KNN kernel (reset by the eigensolver)
     unsigned pad[42];
@@ -215,6 +215,11 @@ cudaError_t launch_batch_svm_knn(const BatchFrame *frames, const PixItem *items,
 // n_vec > 1 (with s.vk, s.lamk, s.vkf set): also the next n_vec - 1 leading
 // eigenvectors, refined the same way (multi-PC projection).
 cudaError_t launch_jacobi(int B, const PcaScratch &s, cudaStream_t st, int n_vec = 1);
+// The leading eigenpair from a Krylov space, the default form up to 256 bands
+// (k_krylov.cu); frames it cannot finish are flagged (Control::jac_redo).
+bool krylov_applies(int B);
+cudaError_t launch_krylov(int B, const PcaScratch &s, cudaStream_t st);
+cudaError_t launch_batch_krylov(const BatchFrame *frames, int n_frames, int B, cudaStream_t st);
 // Kernels launch_jacobi launches for these arguments.
 int jacobi_kernel_count(int B, const PcaScratch &s, int n_vec = 1);
 // The first Jacobi sweep on a thread-block cluster (129 <= B <= 256): its

@@ -1,5 +1,8 @@
 // Step (iii) of the PCA (Section II.C.2, III.A.2.c): Jacobi eigen-decomposition
-// of the B x B covariance, leading eigenvector kept.
+// of the B x B covariance, leading eigenvector kept. This kernel serves more
+// than 256 bands, the plain form (HSC_JACOBI_ONE_CTA), the further eigenvectors
+// of the multi-PC projection, and the frames that the Krylov form (k_krylov.cu,
+// the default up to 256 bands) leaves to it.
 //
 // GB300 design (one CTA, the matrix never leaves the SM):
 //  1. One sweep of parallel cyclic Jacobi in FP32 on A = C / max diag: each
@@ -65,9 +68,12 @@ struct JacParams {
     // 1: the basis from one Jacobi sweep even where block power steps would
     // give it (B <= 128)
     int sweep_basis;
-    // 1: run only for a frame the lean form left (Control::jac_redo), then
+    // 1: run only for a frame the Krylov form left (Control::jac_redo), then
     // clear the flag
     int only_if_flagged;
+    // 1 (several eigenvectors): unless the Krylov form left the frame, v1 is
+    // its and only the further ones are found here
+    int keep_lead;
 };
 
 // j-slices of the double-float C v: each thread sums at most 16 products
@@ -199,13 +205,7 @@ __device__ float block_sumf(float v, float *red)
     return t;
 }
 
-// kLean: the default form for up to 128 bands in shared memory with one
-// eigenvector, compiled without the sweeps, the rebuilds, the fallback and
-// the further eigenvectors, so that its short serial phases stay in the
-// instruction cache (the full kernel spent several cycles per issue waiting
-// for instructions); a frame it cannot finish (a zero C, or a refinement
-// that does not converge) it flags for the full kernel launched after it.
-template <bool kPacked, bool kBatch = false, bool kLean = false>
+template <bool kPacked, bool kBatch = false>
 __global__ void __launch_bounds__(kJacThreads, 1)
 jacobi_kernel(JacParams prm, const double *__restrict__ C, const float2 *__restrict__ C2,
               const double *__restrict__ mu,
@@ -224,7 +224,9 @@ jacobi_kernel(JacParams prm, const double *__restrict__ C, const float2 *__restr
         muf = fr.muf;
         ctl = fr.ctl;
     }
-    if (prm.only_if_flagged && *(volatile unsigned *)&ctl->jac_redo == 0u) return;  // uniform
+    const bool flagged = *(volatile unsigned *)&ctl->jac_redo != 0u;  // uniform
+    if (prm.only_if_flagged && !flagged) return;
+    const bool kept = prm.keep_lead && !flagged;
     extern __shared__ float smem[];
     const int B = prm.B, n = prm.n, P = n / 2;
     const int ld = n + 1;  // odd row stride: column walks hit distinct banks
@@ -299,9 +301,7 @@ jacobi_kernel(JacParams prm, const double *__restrict__ C, const float2 *__restr
                            P <= kPosMaxP && nno <= 2 * (nthr - OW) + OW;
     // Rayleigh-Ritz on the basis (below): the shared-memory form, B <= 128
     const bool ritz = !kPacked && prm.use_smem && B <= 128 && (pos_sweep || presweep || power);
-    if constexpr (!kLean) {
-        if (!pos_sweep && !presweep && !power) load_A();  // sweep_pos loads its own blocks
-    }
+    if (!pos_sweep && !presweep && !power) load_A();  // sweep_pos loads its own blocks
     __syncthreads();
 
     // Work items fixed for the whole run: up to kBlk off-diagonal 2x2 blocks
@@ -342,7 +342,7 @@ jacobi_kernel(JacParams prm, const double *__restrict__ C, const float2 *__restr
     for (int b = 0; b < kBlk; ++b) {
         const int g = tid + b * nthr;
         slot[b] = -1;
-        if (kLean || !blocks_in_regs || g >= nblk) continue;
+        if (!blocks_in_regs || g >= nblk) continue;
         int k, l, o = -1;
         if (!one_sync) {
             tri_of(g, P - 1, k, l);
@@ -839,19 +839,13 @@ jacobi_kernel(JacParams prm, const double *__restrict__ C, const float2 *__restr
     // ---- phase 0: the basis (block power steps, or one logged sweep and the
     // rebuilt leading columns), Rayleigh-Ritz, refinement
     long long t0 = clock64();
-    if constexpr (kLean) {
-        if (!power) {  // a zero C: the full kernel takes the frame
-            if (tid == 0) ctl->jac_redo = 1u;
-            return;
-        }
-    }
     if (power) {  // C's diagonal in the units of A
         stage_c();
         __syncthreads();
         const float2 *Cp = reinterpret_cast<const float2 *>(smem);
         for (int j = tid; j < B; j += nthr) sr[j] = Cp[(size_t)j * B + j].x * inv_p2;
         __syncthreads();
-    } else if constexpr (!kLean) {
+    } else {
         if (presweep) {  // the diagonal after the cluster's sweep (same scaling)
             const float *dg = prm.pre + (size_t)kBasis * prm.pre_n;
             for (int j = tid; j < B; j += nthr) sr[j] = dg[j];
@@ -897,7 +891,7 @@ jacobi_kernel(JacParams prm, const double *__restrict__ C, const float2 *__restr
             for (int ii = lane; ii < n; ii += 32)
                 x[ii] = ii < B ? Cp[(size_t)ii * B + j0].x * inv_p2 : 0.f;
         }
-    } else if constexpr (!kLean) {
+    } else {
 if (presweep) {
         for (int c = warp; c < m; c += nwarps) {
             const float *src = prm.pre + (size_t)c * prm.pre_n;
@@ -1243,25 +1237,22 @@ if (presweep) {
         ts = block_sumf(ts, fred);
         theta_c = (tr - ts) / (float)(B - m);
     }
-    if (prm.use_smem && !kPacked) {
+    if (kept) {
+        refine_iters = 0;  // the lead is k_krylov.cu's
+    } else if (prm.use_smem && !kPacked) {
         // the same pointers, formed from the shared array itself so that
         // the refinement's accesses compile to shared-memory instructions
         const size_t xo = jac_phase0_floats(n);
         refine_iters = refine(smem + xo, m, 0, deflate, theta_c, reinterpret_cast<const float2 *>(smem),
                               reinterpret_cast<float2 *>(smem + xo + (size_t)kBasis * ld));
-    } else if constexpr (!kLean) {
+    } else {
         refine_iters = refine(X, m, 0, deflate, theta_c, prm.use_smem ? Cs2 : C2, part);
     }
     converged = refine_iters <= kMaxRefine;
     t_refine += clock64() - t1;
 
     // ---- fallback: sweeps from C with V accumulated, refinement on all columns
-    if constexpr (kLean) {
-        if (!converged) {  // the full kernel takes the frame
-            if (tid == 0) ctl->jac_redo = 1u;
-            return;
-        }
-    } else if (!converged) {
+    if (!converged) {
         fell_back = true;
         t0 = clock64();
         load_A();
@@ -1346,7 +1337,7 @@ if (presweep) {
             if (vfout) vfout[ii] = (float)v;
         }
     };
-    finish(v1_out, v1f, lambda1_out);
+    if (!kept) finish(v1_out, v1f, lambda1_out);
     if (prm.n_vec > 1) {  // row 0 of the multi-PC output is v1
         for (int ii = tid; ii < B; ii += nthr) {
             prm.vk[ii] = v1_out[ii];
@@ -1354,8 +1345,9 @@ if (presweep) {
         }
         if (tid == 0) prm.lamk[0] = *lambda1_out;
     }
-    for (int ii = tid; ii < B; ii += nthr) muf[ii] = (float)mu[ii];
-    if (tid == 0) {
+    if (!kept)
+        for (int ii = tid; ii < B; ii += nthr) muf[ii] = (float)mu[ii];
+    if (tid == 0 && !kept) {
         if (!converged) atomicOr(&ctl->status, ST_NOT_CONVERGED);
         ctl->jacobi_sweeps = (unsigned)sweeps;
         ctl->refine_iters = (unsigned)(refine_iters > kMaxRefine ? kMaxRefine : refine_iters);
@@ -1373,7 +1365,7 @@ if (presweep) {
     // largest diagonal's column after the sweep) by the same deflated
     // correction aimed at column j, then the same sign rule. Phase 0's basis
     // only (the fallback rebuilds none).
-    if (!kLean && prm.n_vec > 1 && !fell_back) {
+    if (prm.n_vec > 1 && !fell_back) {
         const bool sm_basis = prm.use_smem && !kPacked;
         const size_t xo = jac_phase0_floats(n);
         const float *bas = sm_basis ? smem + xo : X;
@@ -1445,23 +1437,16 @@ JacParams jac_params(int B)
     prm.pre_n = 0;
     prm.sweep_basis = 0;
     prm.only_if_flagged = 0;
+    prm.keep_lead = 0;
     return prm;
 }
 }  // namespace
 
-// The lean form serves frames of up to 128 bands whose work area sits in
-// shared memory, for one eigenvector, unless the plain form is asked for.
-bool lean_applies(const JacParams &prm, int n_vec, bool plain)
-{
-    return prm.use_smem && prm.B <= 128 && n_vec <= 1 && !plain;
-}
-
 int jacobi_kernel_count(int B, const PcaScratch &s, int n_vec)
 {
-    const JacParams prm = jac_params(B);
-    if (lean_applies(prm, n_vec, s.jac_plain)) return 2;  // lean + the guarded full kernel
-    if (s.jac_V && !s.jac_plain && jacobi_cluster_floats(B) && jacobi_cluster_usable(B)) return 2;
-    return 1;
+    if (s.jac_plain || !krylov_applies(B)) return 1;
+    if (n_vec <= 1) return 2;  // the Krylov form + the guarded full kernel
+    return s.jac_V && jacobi_cluster_floats(B) && jacobi_cluster_usable(B) ? 3 : 2;
 }
 
 cudaError_t launch_jacobi(int B, const PcaScratch &s, cudaStream_t st, int n_vec)
@@ -1476,25 +1461,18 @@ cudaError_t launch_jacobi(int B, const PcaScratch &s, cudaStream_t st, int n_vec
     const bool packed = !prm.use_smem && need_packed <= kJacSmemLimit;
     if (!prm.use_smem && !s.jac_A) return cudaErrorInvalidValue;
     prm.sweep_basis = s.jac_plain ? 1 : 0;
-    if (lean_applies(prm, prm.n_vec, s.jac_plain)) {
-        // the lean form, then the full kernel for a frame it flagged (the
-        // basis from one sweep; it exits at once otherwise)
-        if (need > 48 * 1024) {
-            cudaFuncSetAttribute(jacobi_kernel<false, false, true>,
-                                 cudaFuncAttributeMaxDynamicSharedMemorySize, (int)need);
-            cudaFuncSetAttribute(jacobi_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)need);
+    if (!s.jac_plain && krylov_applies(B)) {
+        const cudaError_t e = launch_krylov(B, s, st);
+        if (e != cudaSuccess) return e;
+        if (prm.n_vec <= 1) {  // the full kernel for a frame it flagged (else it exits at once)
+            prm.sweep_basis = 1;
+            prm.only_if_flagged = 1;
+        } else {
+            prm.keep_lead = 1;
         }
-        jacobi_kernel<false, false, true><<<1, kJacThreads, need, st>>>(
-            prm, s.C, s.C2, s.mu, s.v1, s.lambda1, s.v1f, s.muf, s.jac_A, s.ctl, nullptr);
-        JacParams full = prm;
-        full.sweep_basis = 1;
-        full.only_if_flagged = 1;
-        jacobi_kernel<false><<<1, kJacThreads, need, st>>>(full, s.C, s.C2, s.mu, s.v1, s.lambda1,
-                                                           s.v1f, s.muf, s.jac_A, s.ctl, nullptr);
-        return cudaGetLastError();
     }
-    if (s.jac_V && !s.jac_plain && jacobi_cluster_floats(B) && jacobi_cluster_usable(B)) {
+    if (prm.n_vec > 1 && s.jac_V && !s.jac_plain && jacobi_cluster_floats(B) &&
+        jacobi_cluster_usable(B)) {
         // the first sweep on a cluster; this kernel continues from its V
         const cudaError_t e = launch_jacobi_cluster(B, s.C2, s.jac_V, s.ctl, prm.rot_tol, st);
         if (e != cudaSuccess) return e;
@@ -1524,15 +1502,12 @@ cudaError_t launch_batch_jacobi(const BatchFrame *frames, int n_frames, int B, c
     const JacParams prm = jac_params(B);
     const size_t need = jac_work_floats(prm.n) * sizeof(float);
     if (!prm.use_smem || n_frames < 1 || B > 128) return cudaErrorInvalidValue;
-    // the lean form per frame, then the full kernel for the frames it flagged
-    if (need > 48 * 1024) {
-        cudaFuncSetAttribute(jacobi_kernel<false, true, true>,
-                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)need);
+    // the Krylov form per frame, then the full kernel for the frames it flagged
+    const cudaError_t e = launch_batch_krylov(frames, n_frames, B, st);
+    if (e != cudaSuccess) return e;
+    if (need > 48 * 1024)
         cudaFuncSetAttribute(jacobi_kernel<false, true>,
                              cudaFuncAttributeMaxDynamicSharedMemorySize, (int)need);
-    }
-    jacobi_kernel<false, true, true><<<n_frames, kJacThreads, need, st>>>(
-        prm, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, frames);
     JacParams full = prm;
     full.sweep_basis = 1;
     full.only_if_flagged = 1;

@@ -1,7 +1,8 @@
 // Step (iii) of the PCA (Section II.C.2, III.A.2.c): the first sweep of the
 // Jacobi eigen-decomposition spread over a thread-block cluster.
 //
-// The one-CTA eigensolver moves every entry of A through one SM's shared
+// It gives the multi-PC projection its basis for 129-256 bands. The one-CTA
+// eigensolver moves every entry of A through one SM's shared
 // memory each round of its first sweep; for 96-256 bands that sweep is most
 // of the eigensolver's time. Here the same sweep (the same round-robin
 // pairing, the same Schur rotations, a pair's own 2x2 block in closed form)
