@@ -82,7 +82,9 @@ typedef struct {
  *               HSC_KNN_SEARCH_HEAP keys every window candidate and keeps the
  *               K smallest in a max-heap (the paper's partial heapsort,
  *               Section III.B.3 a; an A/B point, slower);
- *               HSC_KNN_SEARCH_AUTO (0) = PRUNED when lambda > 0, else FULL.
+ *               HSC_KNN_SEARCH_AUTO (0) = PRUNED when lambda > 0, else FULL
+ *               (which without a spatial term, lambda^2 == 0, takes windows of
+ *               up to 16384 candidates by sorting their values).
  * Distance ties are broken by the smaller linear index; K must not exceed the
  * smallest window, min(ceil(R/2), H) * W, or the call returns
  * HSC_ERR_INVALID_ARG. */

@@ -34,6 +34,7 @@
 
 #include "hsc_internal.cuh"
 #include "knn_generic.cuh"
+#include "knn_value.cuh"
 #include "svm_pixel.cuh"
 
 namespace hsc {
@@ -1432,6 +1433,10 @@ cudaError_t launch_knn(const float *I, const float *P, int k, int H, int W, int 
         default: return cudaErrorInvalidValue;
         }
     }
+    // the full search without a spatial term: by order of value, where the
+    // window can be sorted in shared memory
+    if (knn_value_applies(H, W, R, lambda))
+        return launch_knn_value(I, P, k, H, W, K, R, O, labels, nbr, ctl, st);
     if (R <= 8) return launch_rmax<8>(I, P, k, H, W, K, R, lambda, O, labels, nbr, ctl, st);
     if (R <= 16) return launch_rmax<16>(I, P, k, H, W, K, R, lambda, O, labels, nbr, ctl, st);
     return launch_rmax<32>(I, P, k, H, W, K, R, lambda, O, labels, nbr, ctl, st);
