@@ -149,7 +149,7 @@ struct PixItem {
 // Launch parameters that change only the speed of a pass, never its results
 // (an autotuner picks them per frame shape): the tensor-core Gram's TMA
 // staging depth (3 or 4; 0 = default), and the projection/SVM pass's pixels
-// per thread (1 or 4; 0 = 4, with 16-byte loads when the cube allows them)
+// per thread (1 or 4; 0 = by pixels and classes, see launch_project_svm)
 // and CTAs per SM of its grid-stride launch (0 = 8), and the pruned KNN walk's
 // variant (launch_knn).
 struct Tuning {

@@ -1192,7 +1192,7 @@ svm_knn_batch_kernel(const BatchFrame *__restrict__ frames, const PixItem *__res
 {
     constexpr int M = KC * (KC - 1) / 2;
     constexpr int MA = M > 0 ? M : 1;
-    extern __shared__ float sm[];  // the weights, then the warps' KNN tiles and key buffers
+    extern __shared__ __align__(16) float sm[];  // the weights, then the warps' KNN tiles and key buffers
     __shared__ float sbias[MA], sa[MA], sb[MA];
     __shared__ int s_item;
     for (;;) {  // projection/SVM items, a CTA each
@@ -1208,11 +1208,11 @@ svm_knn_batch_kernel(const BatchFrame *__restrict__ frames, const PixItem *__res
         bool bad = false;
         float *Iw = norm ? fr.Iraw : fr.I;
         if (fr.vec)
-            project_svm_groups<KC, 4, true>(fr.cube, B, fr.N, sm, sbias, sa, sb, true,
+            project_svm_groups<KC, 4, true, false, 4>(fr.cube, B, fr.N, sm, sbias, sa, sb, true,
                                             it.g0 + threadIdx.x, it.g1, blockDim.x, Iw, fr.P,
                                             nullptr, couple_f64, lmin, lmax, bad, 0, fr.P4);
         else
-            project_svm_groups<KC, 4, false, true>(fr.cube, B, fr.N, sm, sbias, sa, sb, true,
+            project_svm_groups<KC, 4, false, true, 4>(fr.cube, B, fr.N, sm, sbias, sa, sb, true,
                                                    threadIdx.x, threadIdx.x + 1, 1, Iw, fr.P,
                                                    nullptr, couple_f64, lmin, lmax, bad,
                                                    (long)it.g0 * 4, fr.P4);
@@ -1274,7 +1274,7 @@ cudaError_t launch_batch_svm_knn_kc(const BatchFrame *frames, const PixItem *ite
 {
     constexpr int M = KC * (KC - 1) / 2;
     const int wfl = (int)(walk_smem_bytes(R, max_rows) / sizeof(float));
-    const size_t smem = sizeof(float) * std::max((size_t)B * (M + 2), (size_t)(kSvmThreads / 32) * wfl);
+    const size_t smem = sizeof(float) * std::max((size_t)B * svm_stride(KC), (size_t)(kSvmThreads / 32) * wfl);
     auto kern = svm_knn_batch_kernel<KC>;
     if (smem > 48 * 1024)
         cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);

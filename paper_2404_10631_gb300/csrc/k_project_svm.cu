@@ -44,7 +44,7 @@ project_svm_kernel(const float *__restrict__ cube, int B, long N,
 {
     constexpr int M = KC * (KC - 1) / 2;
     constexpr int MA = M > 0 ? M : 1;
-    extern __shared__ float ws[];
+    extern __shared__ __align__(16) float ws[];
     __shared__ float sbias[MA], sa[MA], sb[MA];
     stage_weights<KC>(B, v1f, muf, w, bias, pa, pb, ws, sbias, sa, sb);
     __syncthreads();
@@ -70,7 +70,7 @@ project_svm_batch_kernel(const BatchFrame *__restrict__ frames, const PixItem *_
 {
     constexpr int M = KC * (KC - 1) / 2;
     constexpr int MA = M > 0 ? M : 1;
-    extern __shared__ float ws[];
+    extern __shared__ __align__(16) float ws[];
     __shared__ float sbias[MA], sa[MA], sb[MA];
     const PixItem it = items[blockIdx.x];
     const BatchFrame &fr = frames[it.frame];
@@ -79,11 +79,11 @@ project_svm_batch_kernel(const BatchFrame *__restrict__ frames, const PixItem *_
     float lmin = INFINITY, lmax = -INFINITY;
     bool bad = false;
     if (fr.vec)
-        project_svm_groups<KC, 4, true>(fr.cube, B, fr.N, ws, sbias, sa, sb, true,
+        project_svm_groups<KC, 4, true, false, 4>(fr.cube, B, fr.N, ws, sbias, sa, sb, true,
                                         it.g0 + threadIdx.x, it.g1, blockDim.x, fr.I, fr.P,
                                         nullptr, couple_f64, lmin, lmax, bad, 0, fr.P4);
     else  // pixels g0 * 4 + t + 256 u of thread t: every load coalesced
-        project_svm_groups<KC, 4, false, true>(fr.cube, B, fr.N, ws, sbias, sa, sb, true,
+        project_svm_groups<KC, 4, false, true, 4>(fr.cube, B, fr.N, ws, sbias, sa, sb, true,
                                                threadIdx.x, threadIdx.x + 1, 1, fr.I, fr.P,
                                                nullptr, couple_f64, lmin, lmax, bad,
                                                (long)it.g0 * 4, fr.P4);
@@ -121,7 +121,7 @@ cudaError_t launch_kc(const float *cube, int B, long N, const float *v1f, const 
                       float4 *P4)
 {
     constexpr int M = KC * (KC - 1) / 2;
-    size_t smem = sizeof(float) * (size_t)B * (M + 2);
+    size_t smem = sizeof(float) * (size_t)B * svm_stride(KC);
     auto kern = project_svm_kernel<KC, PX, kVec>;
     if (smem > 48 * 1024)
         cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -164,6 +164,21 @@ cudaError_t launch_project_svm(const float *cube, int B, long N, const float *v1
 {
     const int k = (probs != nullptr && model != nullptr) ? model->n_classes : 0;
     const bool vec = (N % 4 == 0) && ((reinterpret_cast<uintptr_t>(cube) & 15u) == 0);
+    // Pixels per thread. Few classes: 4 (16-byte loads) or, with 2, 3 or 5, 2;
+    // many: one (15 accumulators per pixel with 6 classes: 4 pixels leave too
+    // few warps). Under 64 K pixels one as well: the threads are what is short.
+    // Measured, 4 / 2 / 1 pixels: 416 x 512 x 128, 4 classes 27.2 / 29.0 / 32.8
+    // us; 1000 x 1000 x 100, 3 classes 72 / 66 / 77; 509 x 401 x 100, 6 classes
+    // 57 / 49 / 43; 416 x 512 x 128, 8 classes 132 / 92 / 76; 200 x 200 x 128, 4
+    // classes 17.2 / 13.2 / 13.1; 48 x 48 x 125, 4 classes 16.0 / 12.1 / 10.4.
+    if (px == 0) px = N < 65536 || k >= 6 ? 1 : 4;
+    if (px == 4 && (k == 2 || k == 3 || k == 5)) px = 2;
+    if (px == 2 && vec)
+        return dispatch_k<2, true>(k, cube, B, N, v1f, muf, I_raw, model, couple_f64, probs,
+                                   svm_labels, ctl, sm_count, st, max_blocks, P4);
+    if (px == 2)
+        return dispatch_k<2, false>(k, cube, B, N, v1f, muf, I_raw, model, couple_f64, probs,
+                                    svm_labels, ctl, sm_count, st, max_blocks, P4);
     if (px == 1)
         return dispatch_k<1, false>(k, cube, B, N, v1f, muf, I_raw, model, couple_f64, probs,
                                     svm_labels, ctl, sm_count, st, max_blocks, P4);
@@ -189,7 +204,7 @@ cudaError_t launch_batch_kc(const BatchFrame *frames, const PixItem *items, int 
                             const hsc_svm_model *m, bool f64, cudaStream_t st)
 {
     constexpr int M = KC * (KC - 1) / 2;
-    const size_t smem = sizeof(float) * (size_t)B * (M + 2);
+    const size_t smem = sizeof(float) * (size_t)B * svm_stride(KC);
     auto kern = project_svm_batch_kernel<KC>;
     if (smem > 48 * 1024)
         cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);

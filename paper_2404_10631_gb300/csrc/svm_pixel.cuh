@@ -18,6 +18,13 @@ namespace {
 // stride).
 constexpr int kSvmThreads = 256;
 
+// Floats per band of the staged weights (w_0 .. w_{M-1}, v1, mu), padded to
+// 16-byte loads.
+__host__ __device__ constexpr int svm_stride(int k)
+{
+    return (k * (k - 1) / 2 + 2 + 3) & ~3;
+}
+
 template <int KC, typename CT>
 __device__ __forceinline__ void couple_solve(const float *r /* M, pair order */, float *p)
 {
@@ -149,9 +156,22 @@ __device__ __forceinline__ void finish_svm_pixel(const float (&acc)[KC * (KC - 1
 // below g_end of PX pixels: group g holds pixels g * PX + u (one 16-byte
 // load per band when kVec, else PX 4-byte loads), or, kStrided, pixels
 // p_base + g + u * kSvmThreads (4-byte loads, each coalesced across the warp).
-// ws holds per band w_0..w_{M-1}, v1, mu. The arithmetic of a pixel does not
+// ws holds svm_stride(KC) floats per band (16-byte aligned): w_0..w_{M-1}, v1,
+// mu. The arithmetic of a pixel does not
 // depend on the grouping or the loads.
-template <int KC, int PX, bool kVec, bool kStrided = false>
+// The loads run kAhead bands ahead: a band's register is reloaded as soon as
+// its values are used, so a thread always has that many loads in flight. (In
+// blocks of 16 bands, loaded and then used, all warps of the one wave waited
+// out the memory's latency once per block. Measured: the projection alone on
+// 416 x 512 x 128 30.4 -> 19.0 us, on 300 x 400 x 200 45 -> 26 us; 256 snapshot
+// frames' projection + SVM 54 + 87 -> 43 + 75 us; with 4 classes on 416 x 512 x
+// 128 the coupling solves after the last band are the rest, 27 us both ways.)
+// Loads in flight per thread in the single-frame launches (kAhead PX registers
+// beside (M + 1) PX accumulators); the batch's kernels, three CTAs of 256
+// threads per SM at 80 registers, take 4.
+constexpr int svm_ahead(int k, int px) { return px == 4 ? 8 : px == 2 ? 16 : (k >= 5 ? 16 : 32); }
+
+template <int KC, int PX, bool kVec, bool kStrided = false, int kAhead = svm_ahead(KC, PX)>
 __device__ __forceinline__ void project_svm_groups(
     const float *__restrict__ cube, int B, long N, const float *ws, const float *sbias,
     const float *sa, const float *sb, bool do_pca, long g_begin, long g_end, long g_step,
@@ -161,7 +181,7 @@ __device__ __forceinline__ void project_svm_groups(
 {
     constexpr int M = KC * (KC - 1) / 2;
     constexpr int MA = M > 0 ? M : 1;
-    constexpr int S = M + 2;
+    constexpr int S = svm_stride(KC);
     constexpr long kPs = kStrided ? kSvmThreads : 1;  // pixel stride within a group
     for (long g = g_begin; g < g_end; g += g_step) {
         const long p0 = kStrided ? p_base + g : g * PX;
@@ -173,33 +193,67 @@ __device__ __forceinline__ void project_svm_groups(
 #pragma unroll
             for (int m = 0; m < MA; ++m) acc[m][u] = 0.f;
         }
-        // deep unrolling keeps many independent loads in flight per thread
-        constexpr int kUnroll = 16;
-#pragma unroll kUnroll
-        for (int b = 0; b < B; ++b) {
-            float x[PX];
+        float x[kAhead][PX];
+        auto load = [&](float (&v)[PX], int b) {
             const float *src = cube + (size_t)b * (size_t)N + p0;
             if constexpr (PX == 4 && kVec) {
-                float4 v = __ldcs(reinterpret_cast<const float4 *>(src));
-                x[0] = v.x;
-                x[1] = v.y;
-                x[2] = v.z;
-                x[3] = v.w;
+                const float4 q = __ldcs(reinterpret_cast<const float4 *>(src));
+                v[0] = q.x;
+                v[1] = q.y;
+                v[2] = q.z;
+                v[3] = q.w;
+            } else if constexpr (PX == 2 && kVec) {
+                const float2 q = __ldcs(reinterpret_cast<const float2 *>(src));
+                v[0] = q.x;
+                v[1] = q.y;
             } else {
 #pragma unroll
                 for (int u = 0; u < PX; ++u)
-                    x[u] = (p0 + u * kPs < N) ? __ldcs(src + u * kPs) : 0.f;
+                    v[u] = (p0 + u * kPs < N) ? __ldcs(src + u * kPs) : 0.f;
             }
-            const float *wr = ws + b * S;
+        };
+        auto use = [&](const float (&v)[PX], int b) {
+            float wr[S];
+            const float4 *w4 = reinterpret_cast<const float4 *>(ws + b * S);
 #pragma unroll
-            for (int m = 0; m < M; ++m) {
-                float wm = wr[m];
-#pragma unroll
-                for (int u = 0; u < PX; ++u) acc[m][u] = fmaf(wm, x[u], acc[m][u]);
+            for (int i = 0; i < S / 4; ++i) {
+                const float4 q = w4[i];
+                wr[4 * i] = q.x;
+                wr[4 * i + 1] = q.y;
+                wr[4 * i + 2] = q.z;
+                wr[4 * i + 3] = q.w;
             }
-            const float vb = wr[M], mb = wr[M + 1];
 #pragma unroll
-            for (int u = 0; u < PX; ++u) accI[u] = fmaf(vb, x[u] - mb, accI[u]);
+            for (int m = 0; m < M; ++m)
+#pragma unroll
+                for (int u = 0; u < PX; ++u) acc[m][u] = fmaf(wr[m], v[u], acc[m][u]);
+#pragma unroll
+            for (int u = 0; u < PX; ++u) accI[u] = fmaf(wr[M], v[u] - wr[M + 1], accI[u]);
+        };
+#pragma unroll
+        for (int i = 0; i < kAhead; ++i)
+            if (i < B) load(x[i], i);
+        int b = 0;
+#pragma unroll 1
+        for (; b + 2 * kAhead <= B; b += kAhead) {
+#pragma unroll
+            for (int i = 0; i < kAhead; ++i) {
+                use(x[i], b + i);
+                load(x[i], b + i + kAhead);
+            }
+        }
+        // the last bands: fewer than kAhead still to load
+#pragma unroll
+        for (int i = 0; i < kAhead; ++i) {
+            if (b + i >= B) break;
+            use(x[i], b + i);
+            if (b + i + kAhead < B) load(x[i], b + i + kAhead);
+        }
+        b += kAhead;
+#pragma unroll
+        for (int i = 0; i < kAhead; ++i) {
+            if (b + i >= B) break;
+            use(x[i], b + i);
         }
 #pragma unroll
         for (int u = 0; u < PX; ++u) {
@@ -225,15 +279,22 @@ __device__ __forceinline__ void stage_weights(int B, const float *__restrict__ v
                                               float *sbias, float *sa, float *sb)
 {
     constexpr int M = KC * (KC - 1) / 2;
-    constexpr int S = M + 2;
+    constexpr int S = svm_stride(KC);
     const bool do_pca = (v1f != nullptr);
-    for (int idx = threadIdx.x; idx < B * S; idx += blockDim.x) {
-        int b = idx / S, m = idx % S;
-        float v;
-        if (m < M) v = w[(size_t)m * B + b];
-        else if (m == M) v = do_pca ? v1f[b] : 0.f;
-        else v = do_pca ? muf[b] : 0.f;
-        ws[idx] = v;
+    // a band per thread: its rows' loads go together, each coalesced over bands
+    for (int b = threadIdx.x; b < B; b += blockDim.x) {
+        float v[S];
+#pragma unroll
+        for (int m = 0; m < S; ++m)
+            v[m] = m < M ? w[(size_t)m * B + b] : 0.f;
+        if (do_pca) {
+            v[M] = v1f[b];
+            v[M + 1] = muf[b];
+        }
+        float4 *dst = reinterpret_cast<float4 *>(ws + b * S);
+#pragma unroll
+        for (int i = 0; i < S / 4; ++i)
+            dst[i] = make_float4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
     }
     if constexpr (M > 0)
         for (int m = threadIdx.x; m < M; m += blockDim.x) {
