@@ -111,7 +111,7 @@ typedef struct {
 /* flag for hsc_pca_covariance / hsc_classify */
 #define HSC_COV_FP32_PIPE 4u     /* compute the Gram on the FP32 pipe instead of the tensor cores */
 /* flags for hsc_svm_probs / hsc_classify */
-#define HSC_SVM_COUPLE_F64 2u    /* solve the per-pixel coupling system in FP64 */
+#define HSC_SVM_COUPLE_F64 2u    /* solve the per-pixel coupling system to FP64-level accuracy */
 /* flag for hsc_classify / hsc_classify_batch / server requests: the KNN runs
  * on the raw projection I instead of (I - min I)/(max I - min I) (a method
  * variant; one_band then receives the raw I) */

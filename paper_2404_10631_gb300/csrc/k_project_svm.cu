@@ -12,7 +12,8 @@
 // Q_ij = -r_ji r_ij. Q is only positive semi-definite, but Q + e e^T is
 // positive definite and (Q + e e^T) y = e gives p = y / sum(y), so an LDL^T
 // factorisation without pivoting solves it (FP32 by default; its condition
-// number is below ~25 for r in [1e-7, 1-1e-7], FP64 on request).
+// number is below ~25 for r in [1e-7, 1-1e-7]; on request corrected to
+// FP64-level accuracy, couple_solve).
 // The block min/max of I feeds the min-max normalisation.
 #include <cuda_runtime.h>
 #include <math.h>
