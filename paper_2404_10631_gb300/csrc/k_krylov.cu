@@ -2,7 +2,7 @@
 // eigenvector and up to 256 bands: the leading eigenpair of the covariance
 // from a Krylov space, refined in double-float.
 //
-//  1. kSteps steps of Lanczos in FP32 on A = C / 2^e, each new vector made
+//  1. Up to kSteps steps of Lanczos in FP32 on A = C / 2^e, each new vector made
 //     orthogonal to all before it by classical Gram-Schmidt applied twice: a
 //     basis Q and the tridiagonal T = Q^T A Q. The start vector is A's column
 //     of the largest diagonal entry plus 1% of a fixed pseudo-random vector
@@ -35,13 +35,14 @@
 // same decisions. A batch runs the one-CTA form with the same arithmetic, a
 // CTA per frame.
 //
-// Bound: latency (a chain of about 70 block-wide phases). The eigensolver
-// stage, this kernel and the guarded one behind it, measured: 416 x 512 x 128
-// 33.8 us (a block power step, Gram-Schmidt of 16 columns, Rayleigh-Ritz by
-// Jacobi and 5 corrections in one CTA: 87 us); 1024 x 1024 x 256 38 us (one
-// Jacobi sweep on a 16-CTA cluster, then 10-25 corrections on one CTA: 498 us);
-// 300 x 400 x 200 38 us (450 us, and 3.5 ms for frames whose one-sweep basis
-// did not converge).
+// Bound: latency (a chain of about 50 block-wide phases: 2100 cycles a step,
+// 4400 a correction, 9000 before the first step). The eigensolver stage, this
+// kernel and the guarded one behind it, measured: 416 x 512 x 128 29 us (a
+// block power step, Gram-Schmidt of 16 columns, Rayleigh-Ritz by Jacobi and 5
+// corrections in one CTA: 87 us; always 10 steps here: 34 us); 1024 x 1024 x 256
+// 29 us (one Jacobi sweep on a 16-CTA cluster, then 10-25 corrections on one
+// CTA: 498 us); 300 x 400 x 200 29 us (450 us, and 3.5 ms for frames whose
+// one-sweep basis did not converge).
 #include <cuda_runtime.h>
 #include <math.h>
 #include <stdint.h>
@@ -80,7 +81,7 @@ struct Smem {
     static constexpr int kPad = Shape<CL>::kPad;
     float Q[kSteps][kPad];
     float vh[kPad], vl[kPad];
-    float y[kPad], r[kPad];
+    float y[2][kPad], r[kPad];  // y: Lanczos, two steps' buffers
     float2 part[Shape<CL>::kSlices][Shape<CL>::kRows];
     float2 x[2][kPad];  // the exchanged product, two steps' buffers
     float al[kSteps], be[kSteps];
@@ -135,11 +136,20 @@ __device__ __forceinline__ void cluster_barrier()
     asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
-__device__ __forceinline__ void store_peer(const void *local, uint32_t rank, float2 v)
+__device__ __forceinline__ uint32_t peer_addr(const void *local, uint32_t rank)
 {
     const uint32_t a = (uint32_t)__cvta_generic_to_shared(local);
     uint32_t p;
     asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(p) : "r"(a), "r"(rank));
+    return p;
+}
+__device__ __forceinline__ void store_peer(const void *local, uint32_t rank, float v)
+{
+    asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(peer_addr(local, rank)), "f"(v) : "memory");
+}
+__device__ __forceinline__ void store_peer(const void *local, uint32_t rank, float2 v)
+{
+    const uint32_t p = peer_addr(local, rank);
     asm volatile("st.shared::cluster.v2.f32 [%0], {%1, %2};" ::"r"(p), "f"(v.x), "f"(v.y) : "memory");
 }
 
@@ -184,6 +194,18 @@ krylov_kernel(int B, EigFrame fr, const BatchFrame *__restrict__ frames)
     const float2 *__restrict__ C2 = fr.C2;
     const long long t0 = clock64();
 
+    // ---- this thread's part of C: row `row`, columns j0 .. j0 + kNJ - 1 (its
+    // loads are in flight while the diagonal is looked at)
+    const int rl = (warp % Sh::kR) * 32 + lane, row = (int)rank * kRows + rl;
+    const int sl = warp / Sh::kR, j0 = sl * kNJ;
+    float ch[kNJ], cl[kNJ];
+#pragma unroll
+    for (int u = 0; u < kNJ; ++u) {
+        const int j = j0 + u;
+        const float2 c = row < B && j < B ? C2[(size_t)j * B + row] : make_float2(0.f, 0.f);
+        ch[u] = c.x;
+        cl[u] = c.y;
+    }
     // ---- the diagonal: its maximum (the smaller band on ties) and its sum,
     // by every warp alike; A = C / 2^e (exact)
     float dmax, trace;
@@ -218,26 +240,20 @@ krylov_kernel(int B, EigFrame fr, const BatchFrame *__restrict__ frames)
     const float dmax_s = dmax * inv_p2;
     trace *= inv_p2;
 
-    // ---- this thread's part of C: row `row`, columns j0 .. j0 + kNJ - 1
-    const int rl = (warp % Sh::kR) * 32 + lane, row = (int)rank * kRows + rl;
-    const int sl = warp / Sh::kR, j0 = sl * kNJ;
-    float ch[kNJ], cl[kNJ];
 #pragma unroll
     for (int u = 0; u < kNJ; ++u) {
-        const int j = j0 + u;
-        const float2 c = row < B && j < B ? C2[(size_t)j * B + row] : make_float2(0.f, 0.f);
-        ch[u] = c.x * inv_p2;
-        cl[u] = c.y * inv_p2;
+        ch[u] *= inv_p2;
+        cl[u] *= inv_p2;
     }
     // ---- the start vector
     if (tid < kPad) {
         const float g = (float)(((unsigned)tid * 2654435761u >> 16) & 1023u) * (1.f / 512.f) - 1.f;
-        sm.y[tid] = tid < B ? fmaf(0.01f * dmax_s, g, C2[(size_t)jmax * B + tid].x * inv_p2) : 0.f;
+        sm.y[1][tid] = tid < B ? fmaf(0.01f * dmax_s, g, C2[(size_t)jmax * B + tid].x * inv_p2) : 0.f;
     }
     __syncthreads();
     {
-        const float n2 = dot<kPad>(sm.y, sm.y, lane);
-        if (tid < kPad) sm.Q[0][tid] = sm.y[tid] * rsqrtf(n2);
+        const float n2 = dot<kPad>(sm.y[1], sm.y[1], lane);
+        if (tid < kPad) sm.Q[0][tid] = sm.y[1][tid] * rsqrtf(n2);
     }
     __syncthreads();
     if constexpr (CL > 1) cluster_barrier();  // every CTA runs before its memory is written
@@ -258,11 +274,15 @@ krylov_kernel(int B, EigFrame fr, const BatchFrame *__restrict__ frames)
                     s += q.x;
                 }
             }
-            const dfl w = df ? fast_two_sum(s, lo) : dfl{s, 0.f};
-            if constexpr (CL > 1)
-                store_peer(&sm.x[par][(int)rank * kRows + rr], (uint32_t)warp, make_float2(w.h, w.l));
-            else
-                sm.x[par][rr] = make_float2(w.h, w.l);
+            const int at = (int)rank * kRows + rr;
+            if (df) {
+                const dfl w = fast_two_sum(s, lo);
+                if constexpr (CL > 1) store_peer(&sm.x[par][at], (uint32_t)warp, make_float2(w.h, w.l));
+                else sm.x[par][at] = make_float2(w.h, w.l);
+            } else {
+                if constexpr (CL > 1) store_peer(&sm.y[par][at], (uint32_t)warp, s);
+                else sm.y[par][at] = s;
+            }
         }
         if constexpr (CL > 1) cluster_barrier();
         else __syncthreads();
@@ -271,6 +291,7 @@ krylov_kernel(int B, EigFrame fr, const BatchFrame *__restrict__ frames)
     // ---- Lanczos
     const int m = B < kSteps ? B : kSteps;
     int k = 0;
+    float top = 0.f, prod = 1.f;
 #pragma unroll 1
     for (int j = 0;; ++j) {
         {
@@ -288,15 +309,14 @@ krylov_kernel(int B, EigFrame fr, const BatchFrame *__restrict__ frames)
         }
         __syncthreads();
         exchange(false);
-        if (tid < kPad) sm.y[tid] = sm.x[par][tid].x;
+        float *y = sm.y[par];
         par ^= 1;
-        __syncthreads();
         // two passes: the dot products with the columns so far (warp c) and
         // the vector's own square (warp j + 1), then the subtraction
 #pragma unroll 1
         for (int pass = 0; pass < 2; ++pass) {
             if (warp <= j + 1) {
-                const float d = dot<kPad>(warp <= j ? sm.Q[warp] : sm.y, sm.y, lane);
+                const float d = dot<kPad>(warp <= j ? sm.Q[warp] : y, y, lane);
                 if (lane == 0) {
                     if (warp <= j) (pass ? sm.cb : sm.ca)[warp] = d;
                     else sm.n2[pass] = d;
@@ -305,26 +325,32 @@ krylov_kernel(int B, EigFrame fr, const BatchFrame *__restrict__ frames)
             __syncthreads();
             if (pass == 0) {
                 if (tid < kPad) {
-                    float v = sm.y[tid];
+                    float v = y[tid];
 #pragma unroll 4
                     for (int c = 0; c <= j; ++c) v = fmaf(-sm.ca[c], sm.Q[c][tid], v);
-                    sm.y[tid] = v;
+                    y[tid] = v;
                 }
                 __syncthreads();
             }
         }
-        float b2 = sm.n2[1], v = tid < kPad ? sm.y[tid] : 0.f;
+        float b2 = sm.n2[1], v = tid < kPad ? y[tid] : 0.f;
 #pragma unroll 4
         for (int c = 0; c <= j; ++c) {
             const float d = sm.cb[c];
             b2 = fmaf(-d, d, b2);
             if (tid < kPad) v = fmaf(-d, sm.Q[c][tid], v);
         }
-        // the space is exhausted when what is left of the product is rounding
-        const bool last = j == m - 1 || !(b2 > 1e-12f * sm.n2[0]);
+        // The space is exhausted when what is left of the product is rounding,
+        // and large enough when the product of beta / theta (theta by the
+        // largest alpha so far) is: it bounds the leading Ritz vector's last
+        // component, its share of the residual, up to the gaps.
+        const float alpha = sm.ca[j] + sm.cb[j];
+        top = fmaxf(top, alpha);
+        prod *= fminf(1.f, b2 * __fdividef(1.f, top * top));  // squares
+        const bool last = j == m - 1 || !(b2 > 1e-12f * sm.n2[0]) || prod < 1e-24f;
         const float ib = last ? 0.f : rsqrtf(b2);
         if (tid == 0) {
-            sm.al[j] = sm.ca[j] + sm.cb[j];
+            sm.al[j] = alpha;
             sm.be[j] = last ? 0.f : b2 * ib;
         }
         if (last) {
@@ -355,7 +381,7 @@ krylov_kernel(int B, EigFrame fr, const BatchFrame *__restrict__ frames)
         rest = trace - sum;
         hi = hi * (1.f + 1e-6f);
 #pragma unroll 1
-        for (int round = 0; round < 5; ++round) {
+        for (int round = 0; round < 4; ++round) {
             const float x = lo + (hi - lo) * ((float)(lane + 1) * (1.f / 32.f));
             float d = al[0] - x;
             bool above = d < 0.f;
