@@ -40,6 +40,7 @@
 #include <cuda_runtime.h>
 
 #include "hsc_internal.cuh"
+#include "pdl.cuh"
 #include "tma_util.cuh"
 
 namespace hsc {
@@ -341,6 +342,7 @@ gram_tc_kernel(const __grid_constant__ CUtensorMap tmap, const float *__restrict
     constexpr uint32_t kBoxBytes = G::kBoxBytes, kStageBytes = G::kStageBytes;
     constexpr uint32_t kOpBytes = G::kOpBytes;
     extern __shared__ unsigned char smem_raw[];
+    pdl_wait();
     unsigned char *base = reinterpret_cast<unsigned char *>(
         (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
     unsigned char *staging = base;                                 // kStages x 2 boxes
@@ -756,6 +758,7 @@ gram_tc_wide_kernel(const __grid_constant__ CUtensorMap tmap, const float *__res
                     float *__restrict__ sum_part, Control *ctl)
 {
     extern __shared__ unsigned char smem_raw[];
+    pdl_wait();
     unsigned char *stages = reinterpret_cast<unsigned char *>(
         (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
     __shared__ __align__(8) uint64_t full[kWideStages], conv[kWideStages], empty[kWideStages];
@@ -1178,6 +1181,7 @@ gram_tc_items_kernel(const BatchFrame one, const BatchFrame *__restrict__ frames
     constexpr int kUnits = 8 / kParts;  // 8-pixel fp16 units per thread per chunk
     static_assert(kParts >= 2 && kConv == 128 * kParts, "kParts converter threads per band row");
     extern __shared__ unsigned char smem_raw[];
+    pdl_wait();
     unsigned char *base = reinterpret_cast<unsigned char *>(
         (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
     unsigned char *staging = base;
@@ -1476,8 +1480,8 @@ void launch_narrow(const CUtensorMap &map, const float *cube, int B, int Np, lon
     const size_t smem = Cfg<kSt>::kSmem;
     cudaFuncSetAttribute(gram_tc_kernel<k3D, kSt>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                          (int)smem);
-    gram_tc_kernel<k3D, kSt><<<parts, Cfg<kSt>::kThreads, smem, st>>>(
-        map, cube, B, 0, 0, Np, 1, N, total, per, s.shift, s.gram_part, s.sum_part, s.ctl);
+    launch_pdl(gram_tc_kernel<k3D, kSt>, dim3(parts), dim3(Cfg<kSt>::kThreads), smem, st, map, cube, B,
+               0, 0, Np, 1, N, total, per, s.shift, s.gram_part, s.sum_part, s.ctl);
 }
 
 // The cube's tensor map: 3-D {32 pixels, N / 32 groups, B bands} with boxes
@@ -1511,8 +1515,8 @@ void launch_items(const BatchFrame &one, const BatchFrame *frames, const GramIte
     const size_t smem = Cfg<kSt>::kSmem;
     cudaFuncSetAttribute(gram_tc_items_kernel<kSt>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                          (int)smem);
-    gram_tc_items_kernel<kSt><<<grid, Cfg<kSt>::kThreads, smem, st>>>(
-        one, frames, items, cta_items, n_items, B);
+    launch_pdl(gram_tc_items_kernel<kSt>, dim3(grid), dim3(Cfg<kSt>::kThreads), smem, st, one, frames,
+               items, cta_items, n_items, B);
 }
 }  // namespace
 
@@ -1561,8 +1565,8 @@ cudaError_t launch_gram_tc(const float *cube, int B, long N, const PcaScratch &s
     // 128 < B <= 256: one launch, each chunk read and converted once
     cudaFuncSetAttribute(gram_tc_wide_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                          (int)kWideSmem);
-    gram_tc_wide_kernel<<<parts, kWideThreads, kWideSmem, st>>>(
-        map, cube, B, Np, N, total, per, s.shift, s.gram_part, s.sum_part, s.ctl);
+    launch_pdl(gram_tc_wide_kernel, dim3(parts), dim3(kWideThreads), kWideSmem, st, map, cube, B, Np, N,
+               total, per, s.shift, s.gram_part, s.sum_part, s.ctl);
     return cudaGetLastError();
 }
 

@@ -37,6 +37,7 @@
 #include <type_traits>
 
 #include "hsc_internal.cuh"
+#include "pdl.cuh"
 #include "jacobi_rot.cuh"
 #include "dfloat.cuh"
 
@@ -213,6 +214,7 @@ jacobi_kernel(JacParams prm, const double *__restrict__ C, const float2 *__restr
               float *__restrict__ v1f, float *__restrict__ muf, float *gwork, Control *ctl,
               const BatchFrame *__restrict__ frames)
 {
+    pdl_wait();
     if (kBatch) {  // a stage-major batch: one CTA per frame (work area in shared memory)
         const BatchFrame &fr = frames[blockIdx.x];
         C = fr.C;
@@ -225,7 +227,10 @@ jacobi_kernel(JacParams prm, const double *__restrict__ C, const float2 *__restr
         ctl = fr.ctl;
     }
     const bool flagged = *(volatile unsigned *)&ctl->jac_redo != 0u;  // uniform
-    if (prm.only_if_flagged && !flagged) return;
+    if (prm.only_if_flagged && !flagged) {
+        pdl_next();
+        return;
+    }
     const bool kept = prm.keep_lead && !flagged;
     extern __shared__ float smem[];
     const int B = prm.B, n = prm.n, P = n / 2;
@@ -1482,17 +1487,15 @@ cudaError_t launch_jacobi(int B, const PcaScratch &s, cudaStream_t st, int n_vec
     if (packed) {
         cudaFuncSetAttribute(jacobi_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)need_packed);
-        jacobi_kernel<true><<<1, kJacThreads, need_packed, st>>>(
-            prm, s.C, s.C2, s.mu, s.v1, s.lambda1, s.v1f, s.muf, s.jac_A, s.ctl, nullptr);
-        return cudaGetLastError();
+        return launch_pdl(jacobi_kernel<true>, dim3(1), dim3(kJacThreads), need_packed, st, prm, s.C,
+                          s.C2, s.mu, s.v1, s.lambda1, s.v1f, s.muf, s.jac_A, s.ctl, nullptr);
     }
     const size_t smem = prm.use_smem ? need : 0;
     if (smem > 48 * 1024)
         cudaFuncSetAttribute(jacobi_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)smem);
-    jacobi_kernel<false><<<1, kJacThreads, smem, st>>>(prm, s.C, s.C2, s.mu, s.v1, s.lambda1,
-                                                       s.v1f, s.muf, s.jac_A, s.ctl, nullptr);
-    return cudaGetLastError();
+    return launch_pdl(jacobi_kernel<false>, dim3(1), dim3(kJacThreads), smem, st, prm, s.C, s.C2, s.mu,
+                      s.v1, s.lambda1, s.v1f, s.muf, s.jac_A, s.ctl, nullptr);
 }
 
 // Stage-major batch: one CTA per frame, the single-frame launch's parameters

@@ -33,6 +33,7 @@
 #include <vector>
 
 #include "hsc_internal.cuh"
+#include "pdl.cuh"
 #include "knn_generic.cuh"
 #include "knn_value.cuh"
 #include "svm_pixel.cuh"
@@ -992,6 +993,8 @@ knn_redo_kernel(const float *__restrict__ I, const float *__restrict__ P, int H,
                 int32_t *__restrict__ nbr, Control *ctl, const float4 *__restrict__ P4)
 {
     extern __shared__ float sm[];
+    pdl_wait();
+    pdl_next();
     const long N = (long)H * W;
     if (*(volatile unsigned *)&ctl->knn_redo == 0u) return;
     for (long base = (long)blockIdx.x * kRedoThreads; base < N;
@@ -1116,9 +1119,8 @@ cudaError_t launch_pruned(const float *I, const float *P, int H, int W, int K, i
     // completed in parallel; with nothing flagged every CTA exits at once
     const long rgrid = (N + kRedoThreads - 1) / kRedoThreads;
     const long rcap = (long)redo_resident_ctas(rsmem);
-    knn_redo_kernel<KC><<<(unsigned)(rgrid < rcap ? rgrid : rcap), kRedoThreads, rsmem, st>>>(
-        I, P, H, W, K, R, lam, O, labels, nbr, ctl, P4);
-    return cudaGetLastError();
+    return launch_pdl(knn_redo_kernel<KC>, dim3((unsigned)(rgrid < rcap ? rgrid : rcap)),
+                      dim3(kRedoThreads), rsmem, st, I, P, H, W, K, R, lam, O, labels, nbr, ctl, P4);
 }
 
 template <int KC>

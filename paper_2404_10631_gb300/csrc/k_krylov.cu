@@ -48,6 +48,7 @@
 #include <stdint.h>
 
 #include "hsc_internal.cuh"
+#include "pdl.cuh"
 #include "dfloat.cuh"
 
 namespace hsc {
@@ -185,6 +186,7 @@ krylov_kernel(int B, EigFrame fr, const BatchFrame *__restrict__ frames)
     constexpr int kPad = Sh::kPad, kRows = Sh::kRows, kSlices = Sh::kSlices, kNJ = Sh::kNJ;
     constexpr int kVW = kPad / 32;  // warps that hold a vector
     __shared__ __align__(16) Smem<CL> sm;
+    pdl_wait();
     if (kBatch) {
         const BatchFrame &b = frames[blockIdx.x];
         fr = {b.C2, b.mu, b.v1, b.lambda1, b.v1f, b.muf, b.ctl};
@@ -591,21 +593,22 @@ cudaError_t launch_krylov(int B, const PcaScratch &s, cudaStream_t st)
 {
     const EigFrame fr = {s.C2, s.mu, s.v1, s.lambda1, s.v1f, s.muf, s.ctl};
     if (B <= Shape<1>::kPad) {
-        krylov_kernel<1, false><<<1, kThreads, 0, st>>>(B, fr, nullptr);
-        return cudaGetLastError();
+        return launch_pdl(krylov_kernel<1, false>, dim3(1), dim3(kThreads), 0, st, B, fr, nullptr);
     }
     if (!krylov_applies(B)) return cudaErrorInvalidValue;
     cudaLaunchConfig_t cfg = {};
-    cudaLaunchAttribute at[1];
+    cudaLaunchAttribute at[2];
     at[0].id = cudaLaunchAttributeClusterDimension;
     at[0].val.clusterDim.x = 8;
     at[0].val.clusterDim.y = 1;
     at[0].val.clusterDim.z = 1;
+    at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;  // as launch_pdl
+    at[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.gridDim = dim3(8, 1, 1);
     cfg.blockDim = dim3(kThreads, 1, 1);
     cfg.stream = st;
     cfg.attrs = at;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = 2;
     const BatchFrame *none = nullptr;
     return cudaLaunchKernelEx(&cfg, krylov_kernel<8, false>, B, fr, none);
 }

@@ -11,6 +11,7 @@
 #include <math.h>
 
 #include "hsc_internal.cuh"
+#include "pdl.cuh"
 #include "dfloat.cuh"
 
 namespace hsc {
@@ -146,6 +147,8 @@ pilot_shift_kernel(const float *__restrict__ cube, int B, long N, float *__restr
 {
     __shared__ float red[8];
     __shared__ float s_sh;
+    pdl_wait();
+    pdl_next();
     const int b = blockIdx.x;
     pilot_band_block(cube + (size_t)b * (size_t)N, N, B, b, shift, ctl, red, &s_sh);
 }
@@ -155,6 +158,8 @@ __global__ void __launch_bounds__(256)
 pilot_small_kernel(const float *__restrict__ cube, int B, long N, float *__restrict__ shift,
                    Control *ctl)
 {
+    pdl_wait();
+    pdl_next();
     const int b = blockIdx.x * 8 + (threadIdx.x >> 5);
     if (b < B) pilot_band_warp(cube + (size_t)b * (size_t)N, N, B, b, shift, ctl);
 }
@@ -229,6 +234,7 @@ gram_partial_kernel(const float *__restrict__ cube, int B, int Bp, long N,
                     float *__restrict__ sum_part, Control *ctl)
 {
     extern __shared__ float smem[];
+    pdl_wait();
     const int ld = Bp + 4;
     float *Yt = smem;                                 // kGramChunk x ld
     float *sh = smem + kGramChunk * ld;               // Bp
@@ -322,6 +328,8 @@ gram_reduce_kernel(int B, double inv_N, int n_part, const float *__restrict__ gr
                    const float *__restrict__ sum_part, const float *__restrict__ shift,
                    double *__restrict__ mu, double *__restrict__ C, float2 *__restrict__ C2)
 {
+    pdl_wait();
+    pdl_next();
     const int lane = threadIdx.x & 31, slice = threadIdx.x >> 5;
     const long e = (long)blockIdx.x * kRedEntries + lane;
     const long BB = (long)B * B;
@@ -484,10 +492,9 @@ static cudaError_t launch_reductions(int B, long N, int n_part, const PcaScratch
 {
     const double inv_N = 1.0 / (double)N;
     const long BB = (long)B * B;
-    gram_reduce_kernel<<<(unsigned)((BB + kRedEntries - 1) / kRedEntries), kRedEntries * kRedSlices,
-                         0, st>>>(B, inv_N, n_part, s.gram_part, s.sum_part, s.shift, s.mu, s.C,
-                                  s.C2);
-    return cudaGetLastError();
+return launch_pdl(gram_reduce_kernel, dim3((unsigned)((BB + kRedEntries - 1) / kRedEntries)),
+                      dim3(kRedEntries * kRedSlices), 0, st, B, inv_N, n_part, s.gram_part,
+                      s.sum_part, s.shift, s.mu, s.C, s.C2);
 }
 
 // Kernels launch_moments issues: the pilot, the Gram, the reduction.
@@ -500,8 +507,11 @@ int moments_kernel_count(const float *cube, int B, long N, bool force_simt)
 cudaError_t launch_moments(const float *cube, int B, long N, const PcaScratch &s, int sm_count,
                            cudaStream_t st, bool force_simt, int gram_stages)
 {
-    if (N <= kPilotSmall) pilot_small_kernel<<<(B + 7) / 8, 256, 0, st>>>(cube, B, N, s.shift, s.ctl);
-    else pilot_shift_kernel<<<B, 256, 0, st>>>(cube, B, N, s.shift, s.ctl);
+    const cudaError_t pe =
+        N <= kPilotSmall
+            ? launch_pdl(pilot_small_kernel, dim3((B + 7) / 8), dim3(256), 0, st, cube, B, N, s.shift, s.ctl)
+            : launch_pdl(pilot_shift_kernel, dim3(B), dim3(256), 0, st, cube, B, N, s.shift, s.ctl);
+    if (pe != cudaSuccess) return pe;
     if (!force_simt && gram_tc_usable(cube, B, N)) {
         PcaScratch t = s;
         t.n_part = s.n_part < sm_count ? s.n_part : sm_count;  // one CTA per SM
@@ -517,8 +527,10 @@ cudaError_t launch_moments(const float *cube, int B, long N, const PcaScratch &s
         cudaFuncSetAttribute(gram_partial_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)smem);
     dim3 grid(s.n_part, groups);
-    gram_partial_kernel<<<grid, kGramThreads, smem, st>>>(cube, B, Bp, N, s.shift, s.gram_part,
-                                                          s.sum_part, s.ctl);
+    const cudaError_t ge =
+        launch_pdl(gram_partial_kernel, grid, dim3(kGramThreads), smem, st, cube, B, Bp, N, s.shift,
+                   s.gram_part, s.sum_part, s.ctl);
+    if (ge != cudaSuccess) return ge;
     return launch_reductions(B, N, s.n_part, s, st);
 }
 

@@ -19,6 +19,7 @@
 #include <math.h>
 
 #include "hsc_internal.cuh"
+#include "pdl.cuh"
 #include "svm_pixel.cuh"
 
 namespace hsc {
@@ -47,6 +48,7 @@ project_svm_kernel(const float *__restrict__ cube, int B, long N,
     constexpr int MA = M > 0 ? M : 1;
     extern __shared__ __align__(16) float ws[];
     __shared__ float sbias[MA], sa[MA], sb[MA];
+    pdl_wait();
     stage_weights<KC>(B, v1f, muf, w, bias, pa, pb, ws, sbias, sa, sb);
     __syncthreads();
     float lmin = INFINITY, lmax = -INFINITY;
@@ -94,6 +96,8 @@ project_svm_batch_kernel(const BatchFrame *__restrict__ frames, const PixItem *_
 __global__ void normalize_kernel(const float *__restrict__ I_raw, float *__restrict__ I_norm,
                                  long N, const Control *__restrict__ ctl)
 {
+    pdl_wait();
+    pdl_next();
     const float mn = key_to_float(ctl->imin_key), mx = key_to_float(ctl->imax_key);
     const float range = mx - mn;
     for (long p = (long)blockIdx.x * blockDim.x + threadIdx.x; p < N;
@@ -131,10 +135,9 @@ cudaError_t launch_kc(const float *cube, int B, long N, const float *v1f, const 
     long cap = max_blocks > 0 ? (long)max_blocks : (long)sm_count * 8;
     if (blocks > cap) blocks = cap;
     if (blocks < 1) blocks = 1;
-    kern<<<(unsigned)blocks, kFrameThreads, smem, st>>>(
-        cube, B, N, v1f, muf, m ? m->w : nullptr, m ? m->b : nullptr, m ? m->platt_a : nullptr,
-        m ? m->platt_b : nullptr, I_raw, probs, labels, f64 ? 1 : 0, ctl, P4);
-    return cudaGetLastError();
+    return launch_pdl(kern, dim3((unsigned)blocks), dim3(kFrameThreads), smem, st, cube, B, N, v1f, muf,
+                      m ? m->w : nullptr, m ? m->b : nullptr, m ? m->platt_a : nullptr,
+                      m ? m->platt_b : nullptr, I_raw, probs, labels, f64 ? 1 : 0, ctl, P4);
 }
 
 template <int PX, bool kVec>
@@ -195,8 +198,8 @@ cudaError_t launch_normalize(const float *I_raw, float *I_norm, long N, Control 
 {
     long blocks = (N + 255) / 256;
     if (blocks > 65535) blocks = 65535;
-    normalize_kernel<<<(unsigned)blocks, 256, 0, st>>>(I_raw, I_norm, N, ctl);
-    return cudaGetLastError();
+    return launch_pdl(normalize_kernel, dim3((unsigned)blocks), dim3(256), 0, st, I_raw, I_norm, N,
+                      (const Control *)ctl);
 }
 
 namespace {
@@ -250,6 +253,7 @@ __global__ void __launch_bounds__(kThreads)
 project_multi_kernel(const float *__restrict__ cube, int B, long N, const float *__restrict__ vkf,
                      const float *__restrict__ muf, float *__restrict__ out, Control *ctl)
 {
+    pdl_wait();
     constexpr int S = NP + 1;  // per band: v_0..v_{NP-1}, mu
     extern __shared__ float ws[];
     for (int idx = threadIdx.x; idx < B * S; idx += blockDim.x) {

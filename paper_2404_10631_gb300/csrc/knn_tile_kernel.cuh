@@ -41,6 +41,7 @@
 
 #include "hsc_internal.cuh"
 #include "knn_generic.cuh"
+#include "pdl.cuh"
 
 namespace hsc {
 namespace {
@@ -269,6 +270,7 @@ __global__ void __launch_bounds__(32 * kKnnTileMaxWarps)
 knn_tile_kernel(const __grid_constant__ TileArgs a)
 {
     extern __shared__ float sm[];
+    pdl_wait();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
     TileFrame f = a.frame;
     int cta = blockIdx.x, frame = 0;
@@ -349,8 +351,7 @@ cudaError_t launch_tile_kc(const TileArgs &a, int ctas, int warps, cudaStream_t 
     const size_t smem = buf_bytes(kTileCap) * (size_t)warps;
     if (smem > 48 * 1024)
         cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    kern<<<(unsigned)ctas, 32 * warps, smem, st>>>(a);
-    return cudaGetLastError();
+    return launch_pdl(kern, dim3((unsigned)ctas), dim3(32 * warps), smem, st, a);
 }
 
 }  // namespace
