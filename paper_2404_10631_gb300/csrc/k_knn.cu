@@ -1182,13 +1182,13 @@ __device__ bool wait_count(const unsigned *cnt, unsigned target, Control *ctl)
 // outputs are bit-identical to them. kframes: the KNN's frame table (the
 // group's frames, indexed like the redo list); frames: the whole table
 // (the items' frame indices).
-template <int KC>
+template <int KC, bool kF64>
 __global__ void __launch_bounds__(kSvmThreads)
 svm_knn_batch_kernel(const BatchFrame *__restrict__ frames, const PixItem *__restrict__ items,
                      int n_items, const BatchFrame *__restrict__ kframes, int n_kframes,
                      int n_seg, int cta_base, int B, const float *__restrict__ w,
                      const float *__restrict__ bias, const float *__restrict__ pa,
-                     const float *__restrict__ pb, int couple_f64, int K, int R, float lam,
+                     const float *__restrict__ pb, int K, int R, float lam,
                      int norm, int2 *__restrict__ redo_list, unsigned redo_cap, unsigned *claim,
                      int warp_floats)
 {
@@ -1210,13 +1210,13 @@ svm_knn_batch_kernel(const BatchFrame *__restrict__ frames, const PixItem *__res
         bool bad = false;
         float *Iw = norm ? fr.Iraw : fr.I;
         if (fr.vec)
-            project_svm_groups<KC, 4, true, false, 4>(fr.cube, B, fr.N, sm, sbias, sa, sb, true,
+            project_svm_groups<KC, 4, true, kF64, false, 4>(fr.cube, B, fr.N, sm, sbias, sa, sb, true,
                                             it.g0 + threadIdx.x, it.g1, blockDim.x, Iw, fr.P,
-                                            nullptr, couple_f64, lmin, lmax, bad, 0, fr.P4);
+                                            nullptr, lmin, lmax, bad, 0, fr.P4);
         else
-            project_svm_groups<KC, 4, false, true, 4>(fr.cube, B, fr.N, sm, sbias, sa, sb, true,
+            project_svm_groups<KC, 4, false, kF64, true, 4>(fr.cube, B, fr.N, sm, sbias, sa, sb, true,
                                                    threadIdx.x, threadIdx.x + 1, 1, Iw, fr.P,
-                                                   nullptr, couple_f64, lmin, lmax, bad,
+                                                   nullptr, lmin, lmax, bad,
                                                    (long)it.g0 * 4, fr.P4);
         finish_block(true, lmin, lmax, bad, fr.ctl);
         __threadfence();  // this thread's maps and min/max before the count
@@ -1274,10 +1274,9 @@ cudaError_t launch_batch_svm_knn_kc(const BatchFrame *frames, const PixItem *ite
                                     unsigned redo_cap, unsigned *claim, int sm_count,
                                     cudaStream_t st)
 {
-    constexpr int M = KC * (KC - 1) / 2;
     const int wfl = (int)(walk_smem_bytes(R, max_rows) / sizeof(float));
     const size_t smem = sizeof(float) * std::max((size_t)B * svm_stride(KC), (size_t)(kSvmThreads / 32) * wfl);
-    auto kern = svm_knn_batch_kernel<KC>;
+    auto kern = f64 ? svm_knn_batch_kernel<KC, true> : svm_knn_batch_kernel<KC, false>;
     if (smem > 48 * 1024)
         cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     int per = 0;
@@ -1290,7 +1289,7 @@ cudaError_t launch_batch_svm_knn_kc(const BatchFrame *frames, const PixItem *ite
     if (e != cudaSuccess) return e;
     kern<<<(unsigned)grid, kSvmThreads, smem, st>>>(frames, items, n_items, kframes, n_kframes,
                                                     n_seg, cta_base, B, m->w, m->b, m->platt_a,
-                                                    m->platt_b, f64 ? 1 : 0, K, R, lam,
+                                                    m->platt_b, K, R, lam,
                                                     norm ? 1 : 0, redo_list, redo_cap, claim, wfl);
     const size_t rsmem = redo_smem_bytes(K);
     if (rsmem > 48 * 1024)

@@ -34,15 +34,16 @@ constexpr int kFrameThreads = 128;
 
 // KC = 0: projection only. PX = pixels per thread (4, with 16-byte loads
 // when kVec, or 1).
-template <int KC, int PX, bool kVec>
+// kF64: the coupling to FP64-level accuracy (a kernel of its own: the refined
+// solve is several times the code of the plain one).
+template <int KC, int PX, bool kVec, bool kF64>
 __global__ void __launch_bounds__(kThreads)
 project_svm_kernel(const float *__restrict__ cube, int B, long N,
                    const float *__restrict__ v1f, const float *__restrict__ muf,
                    const float *__restrict__ w, const float *__restrict__ bias,
                    const float *__restrict__ pa, const float *__restrict__ pb,
                    float *__restrict__ I_raw, float *__restrict__ probs,
-                   int32_t *__restrict__ labels, int couple_f64, Control *ctl,
-                   float4 *__restrict__ P4)
+                   int32_t *__restrict__ labels, Control *ctl, float4 *__restrict__ P4)
 {
     constexpr int M = KC * (KC - 1) / 2;
     constexpr int MA = M > 0 ? M : 1;
@@ -54,9 +55,9 @@ project_svm_kernel(const float *__restrict__ cube, int B, long N,
     float lmin = INFINITY, lmax = -INFINITY;
     bool bad = false;
     const long ngroups = (N + PX - 1) / PX;
-    project_svm_groups<KC, PX, kVec>(cube, B, N, ws, sbias, sa, sb, v1f != nullptr,
+    project_svm_groups<KC, PX, kVec, kF64>(cube, B, N, ws, sbias, sa, sb, v1f != nullptr,
                                (long)blockIdx.x * blockDim.x + threadIdx.x, ngroups,
-                               (long)gridDim.x * blockDim.x, I_raw, probs, labels, couple_f64,
+                               (long)gridDim.x * blockDim.x, I_raw, probs, labels,
                                lmin, lmax, bad, 0, P4);
     finish_block(v1f != nullptr, lmin, lmax, bad, ctl);
 }
@@ -64,12 +65,11 @@ project_svm_kernel(const float *__restrict__ cube, int B, long N,
 // Stage-major batch: CTA i takes work item i (one frame's groups of 4
 // pixels, 16-byte loads where the frame allows them); labels are not
 // written (the KNN gives them).
-template <int KC>
+template <int KC, bool kF64>
 __global__ void __launch_bounds__(kThreads, 3)
 project_svm_batch_kernel(const BatchFrame *__restrict__ frames, const PixItem *__restrict__ items,
                          int B, const float *__restrict__ w, const float *__restrict__ bias,
-                         const float *__restrict__ pa, const float *__restrict__ pb,
-                         int couple_f64)
+                         const float *__restrict__ pa, const float *__restrict__ pb)
 {
     constexpr int M = KC * (KC - 1) / 2;
     constexpr int MA = M > 0 ? M : 1;
@@ -82,13 +82,13 @@ project_svm_batch_kernel(const BatchFrame *__restrict__ frames, const PixItem *_
     float lmin = INFINITY, lmax = -INFINITY;
     bool bad = false;
     if (fr.vec)
-        project_svm_groups<KC, 4, true, false, 4>(fr.cube, B, fr.N, ws, sbias, sa, sb, true,
+        project_svm_groups<KC, 4, true, kF64, false, 4>(fr.cube, B, fr.N, ws, sbias, sa, sb, true,
                                         it.g0 + threadIdx.x, it.g1, blockDim.x, fr.I, fr.P,
-                                        nullptr, couple_f64, lmin, lmax, bad, 0, fr.P4);
+                                        nullptr, lmin, lmax, bad, 0, fr.P4);
     else  // pixels g0 * 4 + t + 256 u of thread t: every load coalesced
-        project_svm_groups<KC, 4, false, true, 4>(fr.cube, B, fr.N, ws, sbias, sa, sb, true,
+        project_svm_groups<KC, 4, false, kF64, true, 4>(fr.cube, B, fr.N, ws, sbias, sa, sb, true,
                                                threadIdx.x, threadIdx.x + 1, 1, fr.I, fr.P,
-                                               nullptr, couple_f64, lmin, lmax, bad,
+                                               nullptr, lmin, lmax, bad,
                                                (long)it.g0 * 4, fr.P4);
     finish_block(true, lmin, lmax, bad, fr.ctl);
 }
@@ -119,15 +119,13 @@ __global__ void normalize_batch_kernel(const BatchFrame *__restrict__ frames,
         fr.I[p] = (range > 0.f) ? (fr.I[p] - mn) / range : 0.f;
 }
 
-template <int KC, int PX, bool kVec>
+template <int KC, int PX, bool kVec, bool kF64>
 cudaError_t launch_kc(const float *cube, int B, long N, const float *v1f, const float *muf,
-                      float *I_raw, const hsc_svm_model *m, bool f64, float *probs,
-                      int32_t *labels, Control *ctl, int sm_count, cudaStream_t st, int max_blocks,
-                      float4 *P4)
+                      float *I_raw, const hsc_svm_model *m, float *probs, int32_t *labels,
+                      Control *ctl, int sm_count, cudaStream_t st, int max_blocks, float4 *P4)
 {
-    constexpr int M = KC * (KC - 1) / 2;
     size_t smem = sizeof(float) * (size_t)B * svm_stride(KC);
-    auto kern = project_svm_kernel<KC, PX, kVec>;
+    auto kern = project_svm_kernel<KC, PX, kVec, kF64>;
     if (smem > 48 * 1024)
         cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     long groups = (N + PX - 1) / PX;
@@ -137,24 +135,31 @@ cudaError_t launch_kc(const float *cube, int B, long N, const float *v1f, const 
     if (blocks < 1) blocks = 1;
     return launch_pdl(kern, dim3((unsigned)blocks), dim3(kFrameThreads), smem, st, cube, B, N, v1f, muf,
                       m ? m->w : nullptr, m ? m->b : nullptr, m ? m->platt_a : nullptr,
-                      m ? m->platt_b : nullptr, I_raw, probs, labels, f64 ? 1 : 0, ctl, P4);
+                      m ? m->platt_b : nullptr, I_raw, probs, labels, ctl, P4);
 }
 
-template <int PX, bool kVec>
+template <int PX, bool kVec, bool kF64>
 cudaError_t dispatch_k(int k, const float *cube, int B, long N, const float *v1f,
-                       const float *muf, float *I_raw, const hsc_svm_model *m, bool f64,
-                       float *probs, int32_t *labels, Control *ctl, int sm, cudaStream_t st,
-                       int mb, float4 *P4)
+                       const float *muf, float *I_raw, const hsc_svm_model *m, float *probs,
+                       int32_t *labels, Control *ctl, int sm, cudaStream_t st, int mb, float4 *P4)
 {
     switch (k) {
-    case 0: return launch_kc<0, PX, kVec>(cube, B, N, v1f, muf, I_raw, m, f64, probs, labels, ctl, sm, st, mb, P4);
-    case 2: return launch_kc<2, PX, kVec>(cube, B, N, v1f, muf, I_raw, m, f64, probs, labels, ctl, sm, st, mb, P4);
-    case 3: return launch_kc<3, PX, kVec>(cube, B, N, v1f, muf, I_raw, m, f64, probs, labels, ctl, sm, st, mb, P4);
-    case 4: return launch_kc<4, PX, kVec>(cube, B, N, v1f, muf, I_raw, m, f64, probs, labels, ctl, sm, st, mb, P4);
-    case 5: return launch_kc<5, PX, kVec>(cube, B, N, v1f, muf, I_raw, m, f64, probs, labels, ctl, sm, st, mb, P4);
-    case 6: return launch_kc<6, PX, kVec>(cube, B, N, v1f, muf, I_raw, m, f64, probs, labels, ctl, sm, st, mb, P4);
-    case 7: return launch_kc<7, PX, kVec>(cube, B, N, v1f, muf, I_raw, m, f64, probs, labels, ctl, sm, st, mb, P4);
-    case 8: return launch_kc<8, PX, kVec>(cube, B, N, v1f, muf, I_raw, m, f64, probs, labels, ctl, sm, st, mb, P4);
+    case 0:
+        if constexpr (!kF64)
+            return launch_kc<0, PX, kVec, false>(cube, B, N, v1f, muf, I_raw, m, probs, labels, ctl, sm, st, mb, P4);
+        return cudaErrorInvalidValue;
+#define HSC_SVM_K(KC)                                                                               \
+    case KC:                                                                                        \
+        return launch_kc<KC, PX, kVec, kF64>(cube, B, N, v1f, muf, I_raw, m, probs, labels, ctl, sm, \
+                                             st, mb, P4);
+        HSC_SVM_K(2)
+        HSC_SVM_K(3)
+        HSC_SVM_K(4)
+        HSC_SVM_K(5)
+        HSC_SVM_K(6)
+        HSC_SVM_K(7)
+        HSC_SVM_K(8)
+#undef HSC_SVM_K
     default: return cudaErrorInvalidValue;
     }
 }
@@ -177,20 +182,19 @@ cudaError_t launch_project_svm(const float *cube, int B, long N, const float *v1
     // classes 17.2 / 13.2 / 13.1; 48 x 48 x 125, 4 classes 16.0 / 12.1 / 10.4.
     if (px == 0) px = N < 65536 || k >= 6 ? 1 : 4;
     if (px == 4 && (k == 2 || k == 3 || k == 5)) px = 2;
-    if (px == 2 && vec)
-        return dispatch_k<2, true>(k, cube, B, N, v1f, muf, I_raw, model, couple_f64, probs,
-                                   svm_labels, ctl, sm_count, st, max_blocks, P4);
-    if (px == 2)
-        return dispatch_k<2, false>(k, cube, B, N, v1f, muf, I_raw, model, couple_f64, probs,
-                                    svm_labels, ctl, sm_count, st, max_blocks, P4);
-    if (px == 1)
-        return dispatch_k<1, false>(k, cube, B, N, v1f, muf, I_raw, model, couple_f64, probs,
-                                    svm_labels, ctl, sm_count, st, max_blocks, P4);
-    if (vec)
-        return dispatch_k<4, true>(k, cube, B, N, v1f, muf, I_raw, model, couple_f64, probs,
-                                   svm_labels, ctl, sm_count, st, max_blocks, P4);
-    return dispatch_k<4, false>(k, cube, B, N, v1f, muf, I_raw, model, couple_f64, probs,
-                                svm_labels, ctl, sm_count, st, max_blocks, P4);
+    // the refined coupling solves: one or two pixels (its code and registers)
+    if (couple_f64 && k > 0 && px == 4) px = 2;
+#define HSC_SVM_PX(PX, VEC, F64)                                                                   \
+    dispatch_k<PX, VEC, F64>(k, cube, B, N, v1f, muf, I_raw, model, probs, svm_labels, ctl,        \
+                             sm_count, st, max_blocks, P4)
+    if (couple_f64 && k > 0) {
+        if (px == 2) return vec ? HSC_SVM_PX(2, true, true) : HSC_SVM_PX(2, false, true);
+        return HSC_SVM_PX(1, false, true);
+    }
+    if (px == 2) return vec ? HSC_SVM_PX(2, true, false) : HSC_SVM_PX(2, false, false);
+    if (px == 1) return HSC_SVM_PX(1, false, false);
+    return vec ? HSC_SVM_PX(4, true, false) : HSC_SVM_PX(4, false, false);
+#undef HSC_SVM_PX
 }
 
 cudaError_t launch_normalize(const float *I_raw, float *I_norm, long N, Control *ctl,
@@ -203,18 +207,24 @@ cudaError_t launch_normalize(const float *I_raw, float *I_norm, long N, Control 
 }
 
 namespace {
+template <int KC, bool kF64>
+cudaError_t launch_batch_mode(const BatchFrame *frames, const PixItem *items, int n_items, int B,
+                              const hsc_svm_model *m, cudaStream_t st)
+{
+    const size_t smem = sizeof(float) * (size_t)B * svm_stride(KC);
+    auto kern = project_svm_batch_kernel<KC, kF64>;
+    if (smem > 48 * 1024)
+        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    kern<<<n_items, kThreads, smem, st>>>(frames, items, B, m->w, m->b, m->platt_a, m->platt_b);
+    return cudaGetLastError();
+}
+
 template <int KC>
 cudaError_t launch_batch_kc(const BatchFrame *frames, const PixItem *items, int n_items, int B,
                             const hsc_svm_model *m, bool f64, cudaStream_t st)
 {
-    constexpr int M = KC * (KC - 1) / 2;
-    const size_t smem = sizeof(float) * (size_t)B * svm_stride(KC);
-    auto kern = project_svm_batch_kernel<KC>;
-    if (smem > 48 * 1024)
-        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    kern<<<n_items, kThreads, smem, st>>>(frames, items, B, m->w, m->b, m->platt_a, m->platt_b,
-                                          f64 ? 1 : 0);
-    return cudaGetLastError();
+    return f64 ? launch_batch_mode<KC, true>(frames, items, n_items, B, m, st)
+               : launch_batch_mode<KC, false>(frames, items, n_items, B, m, st);
 }
 }  // namespace
 

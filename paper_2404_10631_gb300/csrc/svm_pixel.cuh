@@ -178,12 +178,12 @@ __device__ __forceinline__ void couple_solve(const float *r /* M, pair order */,
 // The end of one pixel's work, common to every form of the pass: I (and its
 // running min/max), the M decision values f = acc + bias, Platt, coupling, the
 // k probabilities, the label and the pixel-interleaved copy.
-template <int KC>
+template <int KC, bool kF64>
 __device__ __forceinline__ void finish_svm_pixel(const float (&acc)[KC * (KC - 1) / 2 > 0 ? KC * (KC - 1) / 2 : 1],
                                              float accI, long p, long N, bool do_pca,
                                              const float *sbias, const float *sa, const float *sb,
                                              float *__restrict__ I_raw, float *__restrict__ probs,
-                                             int32_t *__restrict__ labels, int couple_f64,
+                                             int32_t *__restrict__ labels,
                                              float &lmin, float &lmax, bool &bad,
                                              float4 *__restrict__ P4)
 {
@@ -206,8 +206,7 @@ __device__ __forceinline__ void finish_svm_pixel(const float (&acc)[KC * (KC - 1
             r[m] = fminf(fmaxf(rr, 1e-7f), 1.f - 1e-7f);
         }
         float pr[KC > 0 ? KC : 1];
-        if (couple_f64) couple_solve<KC, true>(r, pr);
-        else couple_solve<KC, false>(r, pr);
+        couple_solve<KC, kF64>(r, pr);
         int best = 0;
         float bv = pr[0];
 #pragma unroll
@@ -251,12 +250,13 @@ __device__ __forceinline__ void finish_svm_pixel(const float (&acc)[KC * (KC - 1
 // threads per SM at 80 registers, take 4.
 constexpr int svm_ahead(int k, int px) { return px == 4 ? 8 : px == 2 ? 16 : (k >= 5 ? 16 : 32); }
 
-template <int KC, int PX, bool kVec, bool kStrided = false, int kAhead = svm_ahead(KC, PX)>
+template <int KC, int PX, bool kVec, bool kF64, bool kStrided = false,
+          int kAhead = svm_ahead(KC, PX)>
 __device__ __forceinline__ void project_svm_groups(
     const float *__restrict__ cube, int B, long N, const float *ws, const float *sbias,
     const float *sa, const float *sb, bool do_pca, long g_begin, long g_end, long g_step,
     float *__restrict__ I_raw, float *__restrict__ probs, int32_t *__restrict__ labels,
-    int couple_f64, float &lmin, float &lmax, bool &bad, long p_base = 0,
+    float &lmin, float &lmax, bool &bad, long p_base = 0,
     float4 *__restrict__ P4 = nullptr)
 {
     constexpr int M = KC * (KC - 1) / 2;
@@ -342,8 +342,8 @@ __device__ __forceinline__ void project_svm_groups(
             float a[MA];
 #pragma unroll
             for (int m = 0; m < MA; ++m) a[m] = acc[m][u];
-            finish_svm_pixel<KC>(a, accI[u], p, N, do_pca, sbias, sa, sb, I_raw, probs, labels,
-                             couple_f64, lmin, lmax, bad, P4);
+            finish_svm_pixel<KC, kF64>(a, accI[u], p, N, do_pca, sbias, sa, sb, I_raw, probs, labels,
+                                       lmin, lmax, bad, P4);
         }
     }
 }
