@@ -16,10 +16,12 @@
 // K <= 64, in the canonical order (the rounding of O does not depend on the
 // path), then picks from the shell in registers.
 //
-// The other pixels (the image's border, whose disks are cut) take box_pixel in
-// CTAs of their own, numbered first; lanes with too large an e_max and border
-// pixels with too many undecided keys are left to the second pass (label
-// kRedoLabel).
+// The other pixels take box_pixel: the image's border, whose disks are cut, in
+// CTAs of their own, numbered first; lanes with too large an e_max in their
+// own warp, a row at a time (left to a second kernel they came to it in
+// clusters, a few warps with several rows each: 509 x 401, K = 24, lambda 0.5
+// 60 us). Pixels with too many undecided keys there are left to the second
+// pass (label kRedoLabel).
 //
 // Measured, walk and second pass together, against one pixel per lane with
 // every candidate of the disk keyed and P gathered by dependent loads:
@@ -165,8 +167,7 @@ __device__ __forceinline__ bool tile_fast(const TileFrame &f, const TileArgs &a,
         }
         const float L = __fmul_rn(l2, (float)a.sK);
         const float Lp = __fmul_rn(l2, (float)a.prev), Ln = __fmul_rn(l2, (float)a.next);
-        auto decided = [&](float vmin, float vmax) {  // (false for NaN or infinite values)
-            const float dI = __fsub_ru(vmax, vmin);
+        auto decided = [&](float dI) {  // (false for NaN or infinite values)
             const float em = __fmul_ru(dI, dI);
             return Ln > __fadd_ru(L, em) && (a.sK == 0 || __fadd_ru(Lp, em) < L);
         };
@@ -176,8 +177,8 @@ __device__ __forceinline__ bool tile_fast(const TileFrame &f, const TileArgs &a,
             vmin = fminf(vmin, __shfl_xor_sync(0xffffffffu, vmin, o));
             vmax = fmaxf(vmax, __shfl_xor_sync(0xffffffffu, vmax, o));
         }
-        ok = decided(vmin, vmax);
-        if (!ok) {  // warp-uniform: each lane over its own columns
+        ok = decided(__fsub_ru(vmax, vmin));
+        if (!ok) {  // warp-uniform: each lane over its own columns, from its own values
             vmin = INFINITY;
             vmax = -INFINITY;
 #pragma unroll 1
@@ -190,7 +191,13 @@ __device__ __forceinline__ bool tile_fast(const TileFrame &f, const TileArgs &a,
                 vmin = fminf(vmin, src < 32 ? a0 : b0);
                 vmax = fmaxf(vmax, src < 32 ? a1 : b1);
             }
-            ok = decided(vmin, vmax);
+            float dI = 0.f;
+#pragma unroll
+            for (int v = 0; v < kV; ++v) {
+                const float Ip = __ldg(f.I + q0 + v * W);
+                dI = fmaxf(dI, fmaxf(__fsub_ru(Ip, vmin), __fsub_ru(vmax, Ip)));
+            }
+            ok = decided(dI);
             if (__ballot_sync(0xffffffffu, ok && on) == 0u) return false;
         }
     }
@@ -301,23 +308,25 @@ knn_tile_kernel(const __grid_constant__ TileArgs a)
     const int K = a.K, W = f.W;
     const TileGeom g = tile_geom(f.H, f.W, a.rad, a.cut, nw);
     unsigned evals = 0, redo = 0;
-    auto leave = [&](int r, int c) {  // to the redo pass
+    auto leave = [&](int p) {  // to the second pass
         ++redo;
-        const int p = r * W + c;
         f.labels[p] = kRedoLabel;
         if (a.frames) {
             const unsigned i = atomicAdd(&a.frames[0].ctl->knn_redo_list, 1u);
             if (i < a.redo_cap) a.redo_list[i] = make_int2(frame, p);
         }
     };
+    // the pixels that box_pixel takes: this lane's border pixel, or the rows
+    // the tile path left (rows first .. first + passes - 1 below p0)
+    int p0 = -1, passes = 0;
     if (cta < g.border_ctas) {
         const long i = (long)cta * blockDim.x + threadIdx.x;
-        int r = 0, c = 0;
-        const bool in = i < g.border_px;
-        if (in) border_pixel(g, f.H, W, a.rad, i, r, c);
-        const unsigned ev = box_pixel<KC, kP4>(f, in ? r * W + c : -1, K, a.R, l2, buf, kTileCap);
-        if (ev != ~0u) evals += ev;
-        else leave(r, c);
+        if (i < g.border_px) {
+            int r, c;
+            border_pixel(g, f.H, W, a.rad, i, r, c);
+            p0 = r * W + c;
+        }
+        passes = 1;
     } else {
         const int t = (cta - g.border_ctas) * nw + warp;
         if (t < g.tiles) {  // warp-uniform
@@ -330,9 +339,16 @@ knn_tile_kernel(const __grid_constant__ TileArgs a)
             const bool on = c >= a.rad && c < W - a.rad;
             const bool fast = tile_fast<KC, kP4>(f, a, r0, c0, lane, on, vfirst, l2);
             if (on && fast) evals += (unsigned)((kV - vfirst) * a.shell);
-            if (on && !fast)
-                for (int v = vfirst; v < kV; ++v) leave(r0 + v, c);
+            if (on && !fast) p0 = (r0 + vfirst) * W + c;
+            passes = __any_sync(0xffffffffu, p0 >= 0) ? kV - vfirst : 0;
         }
+    }
+#pragma unroll 1
+    for (int v = 0; v < passes; ++v) {
+        const int p = p0 >= 0 ? p0 + v * W : -1;
+        const unsigned ev = box_pixel<KC, kP4>(f, p, K, a.R, l2, buf, kTileCap);
+        if (ev != ~0u) evals += ev;
+        else leave(p);
     }
     // the counters: keys formed, pixels left to the second pass
 #pragma unroll
