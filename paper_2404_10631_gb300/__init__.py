@@ -10,7 +10,9 @@ does, and it raises if ``libhsc.so`` has not been built (no CPU fallback).
 from __future__ import annotations
 
 import ctypes
+import itertools
 import os
+import struct
 from typing import Optional
 
 HERE = os.path.dirname(os.path.abspath(__file__))
@@ -76,6 +78,9 @@ class hsc_frame(ctypes.Structure):
     _fields_ = [("cube", ctypes.c_void_p), ("H", ctypes.c_int32), ("W", ctypes.c_int32),
                 ("labels", ctypes.c_void_p), ("out_probs", ctypes.c_void_p),
                 ("one_band", ctypes.c_void_p), ("probs", ctypes.c_void_p)]
+
+
+assert ctypes.sizeof(hsc_frame) == struct.calcsize("=QiiQQQQ")  # hsc_classify_batch packs it
 
 
 class hsc_request(ctypes.Structure):
@@ -195,6 +200,14 @@ def _ptr(t) -> Optional[int]:
     if not t.is_contiguous():
         raise ValueError("expected a contiguous tensor")
     return t.data_ptr()
+
+
+def _ptrs(ts, n: int) -> list:
+    """_ptr of the first n tensors of a list (0 for None)."""
+    if len(ts) < n:
+        raise IndexError("list index out of range")
+    return [t.data_ptr() if t is not None and t.is_cuda and t.is_contiguous() else (_ptr(t) or 0)
+            for t in ts[:n]]
 
 
 class Model:
@@ -459,18 +472,22 @@ def hsc_classify_batch(ctx: Context, cubes, model: Model, K: int, window_rows: i
     label maps (allocated when not given); optional per-frame output lists."""
     import torch
     n = len(cubes)
-    B = int(cubes[0].shape[0])
-    if labels is None:
-        labels = [torch.empty((c.shape[1], c.shape[2]), dtype=torch.int32, device=c.device)
-                  for c in cubes]
-    arr = (hsc_frame * n)()
-    for i, c in enumerate(cubes):
-        if int(c.shape[0]) != B:
+    shapes = [c.shape for c in cubes]
+    B = int(shapes[0][0])
+    for s in shapes:
+        if s[0] != B:
             raise ValueError("all cubes need the same band count")
-        arr[i] = hsc_frame(_ptr(c), int(c.shape[1]), int(c.shape[2]), _ptr(labels[i]),
-                           _ptr(out_probs[i]) if out_probs else None,
-                           _ptr(one_bands[i]) if one_bands else None,
-                           _ptr(probs[i]) if probs else None)
+    if labels is None:
+        labels = [torch.empty((s[1], s[2]), dtype=torch.int32, device=c.device)
+                  for s, c in zip(shapes, cubes)]
+    # the descriptors as one packed block (hsc_frame: cube, H, W, four outputs):
+    # a structure object per frame took longer than the batch on the GPU
+    zeros = [0] * n
+    cols = [_ptrs(cubes, n), [s[1] for s in shapes], [s[2] for s in shapes], _ptrs(labels, n),
+            _ptrs(out_probs, n) if out_probs else zeros,
+            _ptrs(one_bands, n) if one_bands else zeros, _ptrs(probs, n) if probs else zeros]
+    arr = (hsc_frame * n)()
+    struct.pack_into("=" + "QiiQQQQ" * n, arr, 0, *itertools.chain.from_iterable(zip(*cols)))
     ms = model.struct()
     prm = hsc_knn_params(K, window_rows, lam, search)
     ctx.check(lib().hsc_classify_batch(ctx.handle, arr, n, B, ctypes.byref(ms),
