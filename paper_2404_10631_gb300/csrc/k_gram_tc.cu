@@ -1017,40 +1017,6 @@ gram_tc_wide_kernel(const __grid_constant__ CUtensorMap tmap, const float *__res
 
 // ---------------------------------------------------------------- work items
 
-// L2 policy for the cube's chunks: read once, evicted first, so that the
-// partial Grams written meanwhile stay in L2 for the reduction.
-__device__ __forceinline__ uint64_t evict_first_policy()
-{
-    uint64_t pol;
-    asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(pol));
-    return pol;
-}
-
-__device__ __forceinline__ void cp_async4(uint32_t dst, const float *src, bool in, uint64_t pol)
-{
-    asm volatile("cp.async.ca.shared.global.L2::cache_hint [%0], [%1], 4, %2, %3;" ::"r"(dst),
-                 "l"(src), "r"(in ? 4 : 0), "l"(pol)
-                 : "memory");
-}
-
-__device__ __forceinline__ void cp_async16(uint32_t dst, const float *src, bool in, uint64_t pol)
-{
-    asm volatile("cp.async.cg.shared.global.L2::cache_hint [%0], [%1], 16, %2, %3;" ::"r"(dst),
-                 "l"(src), "r"(in ? 16 : 0), "l"(pol)
-                 : "memory");
-}
-
-__device__ __forceinline__ void cp_async_commit()
-{
-    asm volatile("cp.async.commit_group;" ::: "memory");
-}
-
-template <int kPending>
-__device__ __forceinline__ void cp_async_wait()
-{
-    asm volatile("cp.async.wait_group %0;" ::"n"(kPending) : "memory");
-}
-
 // Named barrier of the converter warps that also ORs a predicate over them.
 __device__ __forceinline__ bool conv_bar_or(int nthreads, bool pred)
 {
@@ -1069,49 +1035,129 @@ __device__ __forceinline__ void conv_bar(int nthreads)
     asm volatile("bar.sync 1, %0;" ::"r"(nthreads) : "memory");
 }
 
-// One 64-pixel chunk (pixels p0.., every band row b < B) into a staging slot
-// in the layout a 128-byte-swizzled TMA box would give it (two 32-pixel
-// boxes; in each, band row b at b * 128 with its 16-byte units permuted by
-// b & 7), issued by the kConv converter threads cv: 16-byte copies (row
-// b = f / 16, 4-pixel unit f % 16 for f = cv + kConv i) when the frame allows
-// them, else 4-byte copies (rows cv / 32 + (kConv / 32) i, pixels lane and
-// lane + 32). Pixels at or past N are zero-filled.
-template <uint32_t kBoxBytes, int kConv>
-__device__ __forceinline__ void fetch_chunk(unsigned char *slot, const float *cube, long N,
-                                            bool vec, long p0, int B, int cv)
+// Staging of the work-item form: band row b of a chunk at b * kItemRow, the
+// 16-byte units that hold its 64 pixels wherever they start: 17 of them. (17
+// is odd, so the rows' equal units lie in different banks without a swizzle.)
+constexpr uint32_t kItemRow = 17 * 16;
+constexpr uint32_t kItemStage = 128 * kItemRow;
+constexpr int kItemCopiers = 128;  // threads that copy: warps 0 and 10 - 12
+template <int kSt>
+constexpr int kItemThreads = Cfg<kSt>::kThreads + kItemCopiers - 32;
+template <int kSt>
+constexpr size_t kItemSmem = 1024 + (size_t)kSt * kItemStage +
+                             (size_t)Cfg<kSt>::kOpStages * 2 * Cfg<kSt>::kOpBytes;
+static_assert(kItemStage % 1024 == 0 && kItemSmem<4> <= 227 * 1024,
+              "the operand tiles follow the stages, 1 KB aligned");
+static_assert((size_t)Cfg<>::kRows * kFbLd * 4 <= 3 * (size_t)kItemStage,
+              "the FP32 recompute stages into the ring");
+
+// 16 bytes, of which the first `bytes` are read (the rest become zero).
+__device__ __forceinline__ void cp_async16(uint32_t dst, uint64_t src, uint32_t bytes, uint64_t pol)
 {
-    constexpr int kW = kConv / 32;
-    const uint32_t sbase = smem_u32(slot);
-    const uint64_t pol = evict_first_policy();
-    if (vec) {
+    asm volatile("cp.async.cg.shared.global.L2::cache_hint [%0], [%1], 16, %2, %3;" ::"r"(dst),
+                 "l"(src), "r"(bytes), "l"(pol)
+                 : "memory");
+}
+
+__device__ __forceinline__ void cp_async4(uint32_t dst, uint64_t src)
+{
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(dst), "l"(src) : "memory");
+}
+
+// This thread's arrival on bar once its copies so far have landed.
+__device__ __forceinline__ void cp_async_arrive(uint64_t *bar)
+{
+    asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(smem_u32(bar)) : "memory");
+}
+
+// One 16-byte unit (the u-th from the one that holds the row's first pixel)
+// of the pixels [a, z) of a band row staged at dst; bytes of the cube [lo, hi)
+// only, and nothing past the pixels.
+__device__ __forceinline__ void copy_unit(uint32_t dst, uint64_t a, uint64_t z, uint64_t lo,
+                                          uint64_t hi, uint32_t u, uint64_t pol)
+{
+    const uint64_t at = (a & ~(uint64_t)15) + 16u * u;
+    if (at >= z) return;
+    if (at >= lo) {
+        cp_async16(dst + 16u * u, at, hi - at < 16 ? (uint32_t)(hi - at) : 16u, pol);
+    } else {  // a cube that starts inside a unit: its first floats one by one
+        for (uint32_t i = 0; i < 16; i += 4)
+            if (at + i >= lo && at + i < hi) cp_async4(dst + 16u * u + i, at + i);
+    }
+}
+
+// One 64-pixel chunk (pixels p0.., every band row b < B) into a staging slot,
+// by thread t of the kItemCopiers: units t % 16 of rows t / 16 + 8 i, and the
+// last unit of row t. Eight rows are a multiple of 32 bytes, so all of a
+// thread's rows are aligned alike: away from the frame's ends its copies are
+// one instruction and one addition each. Pixels at or past N keep what the
+// slot held (the conversion zeroes them).
+__device__ __forceinline__ void fetch_chunk(unsigned char *slot, const float *cube, long N,
+                                            long p0, int B, int t, uint64_t pol)
+{
+    constexpr int kStep = kItemCopiers / 16;  // rows between a thread's copies
+    const uint32_t base = smem_u32(slot);
+    const uint64_t lo = (uint64_t)reinterpret_cast<uintptr_t>(cube);
+    const uint64_t row = 4u * (uint64_t)N;
+    const uint32_t u = (uint32_t)t & 15u;
+    const uint64_t a = lo + 4u * (uint64_t)p0 + (uint64_t)(t >> 4) * row;
+    const uint64_t a1 = lo + 4u * (uint64_t)p0 + (uint64_t)t * row;
+    const uint32_t dst = base + (uint32_t)(t >> 4) * kItemRow;
+    const uint32_t dst1 = base + (uint32_t)t * kItemRow;
+    // no unit of these pixels reaches outside its band row
+    if (p0 >= 4 && p0 + kChunk + 4 <= N) {
+        uint64_t src = (a & ~(uint64_t)15) + 16u * u;
 #pragma unroll
-        for (int i = 0; i < 2048 / kConv; ++i) {
-            const int f = cv + kConv * i;
-            const int b = f >> 4, u4 = f & 15;
-            if (b < B) {
-                const long p = p0 + 4 * u4;
-                const bool in = p < N;
-                cp_async16(sbase + (uint32_t)(u4 >> 3) * kBoxBytes + (uint32_t)b * 128u +
-                               (uint32_t)(((u4 & 7) ^ (b & 7)) << 4),
-                           in ? cube + (size_t)b * N + p : cube, in, pol);
-            }
+        for (int i = 0; i < 128 / kStep; ++i) {
+            if ((t >> 4) + i * kStep < B) cp_async16(dst + 16u * u + i * kStep * kItemRow, src, 16u, pol);
+            src += kStep * row;
         }
-    } else {
-        const int w = cv >> 5, lane = cv & 31;
+        if (t < B && (a1 & 15) != 0)
+            cp_async16(dst1 + 256u, (a1 & ~(uint64_t)15) + 256u, 16u, pol);
+        return;
+    }
+    const uint64_t hi = lo + (uint64_t)B * row;
+    const uint64_t n = 4u * (uint64_t)(N - p0 < kChunk ? N - p0 : kChunk);
+    for (int i = 0; (t >> 4) + i * kStep < B; ++i) {
+        const uint64_t ai = a + (uint64_t)(i * kStep) * row;
+        copy_unit(dst + i * kStep * kItemRow, ai, ai + n, lo, hi, u, pol);
+    }
+    if (t < B) copy_unit(dst1, a1, a1 + n, lo, hi, 16u, pol);
+}
+
+// A thread's 32 pixels (units u0 .. u0 + 3 of 8) of a staged band row to the
+// operand tiles, from units that start m floats before the first pixel
+// (kShift; else m = 0): two selects per value.
+template <bool kShift, int kUnits>
+__device__ __forceinline__ void convert_row(const unsigned char *row, int m, float c, float nsc,
+                                            int u0, int sw, bool tail, int lim, unsigned char *ohi,
+                                            unsigned char *olo, float &bsum, float &ymax)
+{
+    const float4 *q = reinterpret_cast<const float4 *>(row) + 2 * u0;
+    float4 next = q[0];
 #pragma unroll
-        for (int i = 0; i < 128 / kW; ++i) {
-            const int b = w + kW * i;
-            if (b < B) {
+    for (int uu = 0; uu < kUnits; ++uu) {
+        const int u = u0 + uu;
+        float4 xa = next, xb = q[2 * uu + 1];
+        if (kShift) {
+            next = q[2 * uu + 2];
+            const float f[12] = {xa.x, xa.y, xa.z, xa.w, xb.x, xb.y, xb.z, xb.w,
+                                 next.x, next.y, next.z, next.w};
+            float t[9], x[8];
 #pragma unroll
-                for (int h = 0; h < 2; ++h) {
-                    const long p = p0 + lane + 32 * h;
-                    const bool in = p < N;
-                    cp_async4(sbase + (uint32_t)h * kBoxBytes + (uint32_t)b * 128u +
-                                  (uint32_t)(((lane >> 2) ^ (b & 7)) << 4) + (uint32_t)(lane & 3) * 4u,
-                              in ? cube + (size_t)b * N + p : cube, in, pol);
-                }
-            }
+            for (int e = 0; e < 9; ++e) t[e] = (m & 2) ? f[e + 2] : f[e];
+#pragma unroll
+            for (int e = 0; e < 8; ++e) x[e] = (m & 1) ? t[e + 1] : t[e];
+            xa = make_float4(x[0], x[1], x[2], x[3]);
+            xb = make_float4(x[4], x[5], x[6], x[7]);
+        } else if (uu + 1 < kUnits) {
+            next = q[2 * uu + 2];
         }
+        uint4 hv, lv;
+        if (tail) convert_unit<true>(xa, xb, c, nsc, u, lim, bsum, ymax, hv, lv);
+        else convert_unit<false>(xa, xb, c, nsc, u, lim, bsum, ymax, hv, lv);
+        *reinterpret_cast<uint4 *>(ohi + ((u ^ sw) << 4)) = hv;
+        *reinterpret_cast<uint4 *>(olo + ((u ^ sw) << 4)) = lv;
     }
 }
 
@@ -1163,12 +1209,20 @@ __device__ __forceinline__ GramItem get_item(const BatchFrame &one,
 // and gets the same partial Gram and sums, bit for bit: the same conversion,
 // MMA sequence, segments and epilogue. With items == nullptr the items are
 // the chunk ranges of the single frame one (one.per chunks each).
-// Warp 1 owns TMEM and issues the MMAs; the 8 converter warps fetch their
-// chunks themselves with asynchronous copies, kSt - 1 chunks ahead, into the
-// staging layout the TMA would write, and one named barrier per chunk among
-// them orders the copies with their readers (and makes every exit uniform).
+// Warps 0 and 10 - 12 copy the chunks, up to kSt ahead and across items; warp 1
+// owns TMEM and issues the MMAs; warps 2 - 9 convert, and meet at named
+// barriers at the ends of an item only.
+// The rows of a frame with N % 4 != 0 start at any float, and a 16-byte copy
+// at a 16-byte boundary: the units around the pixels are copied, and the
+// converters shift what they read. Measured (means and covariance): 1001 x 999
+// x 100 228 -> 153 us, 415 x 513 x 128 68 -> 53 us, 201 x 199 x 100 48 -> 38
+// us against copies of 4 bytes issued by the converters; 256 snapshot frames
+// of 40 - 64 pixels a side, 125 bands, 238 -> 188 us. What is left is the
+// conversion (the copies alone take 93 us of the 153; the shift 12). Bulk
+// copies of a row's 272 bytes instead, by one thread per row: 433 us (some 40
+// ns each).
 template <int kSt>
-__global__ void __launch_bounds__(Cfg<kSt>::kThreads, 1)
+__global__ void __launch_bounds__(kItemThreads<kSt>, 1)
 gram_tc_items_kernel(const BatchFrame one, const BatchFrame *__restrict__ frames,
                      const GramItem *__restrict__ items, const int *__restrict__ cta_items,
                      int n_items, int B)
@@ -1176,7 +1230,6 @@ gram_tc_items_kernel(const BatchFrame one, const BatchFrame *__restrict__ frames
     using G = Cfg<kSt>;
     constexpr int kStages = G::kStages, kOpStages = G::kOpStages, kAccHH = G::kAccHH;
     constexpr int kParts = G::kParts, kConv = 32 * G::kConvWarps;
-    constexpr uint32_t kBoxBytes = G::kBoxBytes, kStageBytes = G::kStageBytes;
     constexpr uint32_t kOpBytes = G::kOpBytes;
     constexpr int kUnits = 8 / kParts;  // 8-pixel fp16 units per thread per chunk
     static_assert(kParts >= 2 && kConv == 128 * kParts, "kParts converter threads per band row");
@@ -1185,8 +1238,8 @@ gram_tc_items_kernel(const BatchFrame one, const BatchFrame *__restrict__ frames
     unsigned char *base = reinterpret_cast<unsigned char *>(
         (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
     unsigned char *staging = base;
-    unsigned char *ops = base + kStages * kStageBytes;
-    __shared__ Bars<kSt> bars;  // full / empty unused: copies complete by groups
+    unsigned char *ops = base + kStages * kItemStage;
+    __shared__ Bars<kSt> bars;
     __shared__ uint32_t tmem_base;
     __shared__ int abort_flag, range_item;
     __shared__ float isc_sh[128], bsum_sh[kParts - 1][128];
@@ -1201,6 +1254,10 @@ gram_tc_items_kernel(const BatchFrame one, const BatchFrame *__restrict__ frames
     (void)n_items;
 
     if (tid == 0) {
+        for (int s = 0; s < kStages; ++s) {
+            mbar_init(&bars.full[s], kItemCopiers);
+            mbar_init(&bars.empty[s], G::kConvWarps);
+        }
         for (int t = 0; t < kOpStages; ++t) {
             mbar_init(&bars.op_full[t], G::kConvWarps);
             mbar_init(&bars.op_empty[t], 1);
@@ -1213,10 +1270,11 @@ gram_tc_items_kernel(const BatchFrame one, const BatchFrame *__restrict__ frames
     }
     const int cv = tid - 64;          // converter index
     const int b0 = cv & 127;          // its band row
-    const int part = cv >> 7;         // which 32-pixel box of a chunk it converts
+    const int part = cv >> 7;         // which 32 pixels of a chunk it converts
     const int sw = b0 & 7;
     const int u0 = part * kUnits;     // its 8-pixel fp16 units
-    if (warp >= 2 && b0 >= B)  // rows beyond B stay zero in every operand stage
+    const bool converter = warp >= 2 && warp < 2 + G::kConvWarps;
+    if (converter && b0 >= B)  // rows beyond B stay zero in every operand stage
         for (int t = 0; t < kOpStages; ++t)
             for (int u = u0; u < u0 + kUnits; ++u) {
                 const uint4 z = make_uint4(0, 0, 0, 0);
@@ -1238,7 +1296,29 @@ gram_tc_items_kernel(const BatchFrame one, const BatchFrame *__restrict__ frames
     volatile int *abort_p = &abort_flag;
     int ncommit = 0;
 
-    if (warp == 1) {
+    if (warp != 1 && !converter) {
+        // ---------------- the copies of every chunk of every item
+        const uint64_t pol = l2_policy_evict_first();
+        const int t = warp == 0 ? tid : tid - G::kThreads + 32;
+        long g = 0;  // chunks so far
+        bool stop = false;
+        for (int it = it_begin; it < it_end && !stop; ++it) {
+            const GramItem item = get_item(one, items, it);
+            const ItemFrame fr = item_frame(one, frames, item.frame);
+            for (int ch = item.c0; ch < item.c1; ++ch, ++g) {
+                const int slot = (int)(g % kStages);
+                if (g >= kStages &&
+                    !__all_sync(0xffffffffu, mbar_wait(&bars.empty[slot],
+                                                       (uint32_t)(((g / kStages) - 1) & 1), abort_p))) {
+                    stop = true;
+                    break;
+                }
+                fetch_chunk(staging + slot * kItemStage, fr.cube, fr.N, (long)ch * kChunk, B, t, pol);
+                cp_async_arrive(&bars.full[slot]);
+            }
+        }
+        asm volatile("cp.async.wait_all;" ::: "memory");
+    } else if (warp == 1) {
         // ---------------- MMA issuer over every chunk of every item
         if (lane == 0) {
             const uint32_t idesc = (1u << 4) | ((uint32_t)(Np >> 3) << 17) | ((uint32_t)(kM >> 4) << 24);
@@ -1276,34 +1356,8 @@ gram_tc_items_kernel(const BatchFrame one, const BatchFrame *__restrict__ frames
                 ++ncommit;
             }
         }
-    } else if (warp >= 2) {
-        // ---------------- converters: copies, conversion, epilogue
-        // prefetch cursor: chunk pf_j of item pf_it
-        int pf_it = it_begin, pf_j = 0, pf_n = 0, pf_c0 = 0;
-        ItemFrame pf{};
-        auto pf_item = [&]() {
-            if (pf_it < it_end) {
-                const GramItem gi = get_item(one, items, pf_it);
-                pf = item_frame(one, frames, gi.frame);
-                pf_c0 = gi.c0;
-                pf_n = gi.c1 - gi.c0;
-            }
-        };
-        auto fetch_next = [&](long slot) {
-            if (pf_it < it_end) {
-                fetch_chunk<kBoxBytes, kConv>(staging + slot * kStageBytes, pf.cube, pf.N,
-                                              pf.vec != 0, (long)(pf_c0 + pf_j) * kChunk, B, cv);
-                if (++pf_j == pf_n) {
-                    pf_j = 0;
-                    ++pf_it;
-                    pf_item();
-                }
-            }
-            cp_async_commit();  // one group per chunk slot, empty past the last chunk
-        };
-        pf_item();
-        for (int k = 0; k < kStages - 1; ++k) fetch_next(k);
-
+    } else {
+        // ---------------- converters: conversion, epilogue
         long g = 0;
         int s = 0;
         bool stop = false;
@@ -1314,49 +1368,43 @@ gram_tc_items_kernel(const BatchFrame one, const BatchFrame *__restrict__ frames
             const float nsc = -(b0 < B ? fr.shift[b0] : 0.f) * c;  // exact: c is a power of two
             if (cv < 128) isc_sh[cv] = __frcp_rn(cv < B ? fr.shift[B + cv] : 1.f);
             if (cv == 0) range_item = 0;
+            conv_bar(kConv);  // isc_sh written
+            // floats before a row's first pixel in its first 16-byte unit
+            const int m = (int)(((reinterpret_cast<uintptr_t>(fr.cube) >> 2) +
+                                 (uintptr_t)b0 * (uintptr_t)fr.N) & 3);
             float *out = fr.gram_part + (size_t)item.part * B * B;
             float bsum = 0.f, ymax = 0.f;
             const int nch = item.c1 - item.c0;
             for (int ji = 0; ji < nch; ++ji, ++g) {
                 const int slot = (int)(g % kStages), t = (int)(g % kOpStages);
-                cp_async_wait<kStages - 2>();  // this thread's copies of chunk g landed
-                bool ok = true;
-                if (g >= kOpStages)
-                    ok = mbar_wait(&bars.op_empty[t], (uint32_t)(((g / kOpStages) - 1) & 1), abort_p);
-                // every converter's copies of chunk g landed and chunk g - 1 is converted
-                if (conv_bar_or(kConv, !ok || *abort_p)) {
+                if (!__all_sync(0xffffffffu, mbar_wait(&bars.full[slot],
+                                                       (uint32_t)((g / kStages) & 1), abort_p)) ||
+                    (g >= kOpStages &&
+                     !__all_sync(0xffffffffu, mbar_wait(&bars.op_empty[t],
+                                                        (uint32_t)(((g / kOpStages) - 1) & 1),
+                                                        abort_p)))) {
                     stop = true;
                     break;
                 }
-                fetch_next((g + kStages - 1) % kStages);
                 const long px0 = (long)(item.c0 + ji) * kChunk;
                 const bool tail = px0 + kChunk > fr.N;
                 const int lim = tail ? (int)(fr.N - px0) : kChunk;
                 if (b0 < B) {
-                    const unsigned char *st = staging + slot * kStageBytes;
+                    const unsigned char *row = staging + slot * kItemStage + b0 * kItemRow;
                     unsigned char *ohi = ops + t * 2 * kOpBytes + b0 * 128;
-                    unsigned char *olo = ohi + kOpBytes;
-#pragma unroll
-                    for (int uu = 0; uu < kUnits; ++uu) {
-                        const int u = u0 + uu;
-                        const int box = u >> 2;
-                        const int j0 = (u & 3) * 2;
-                        const unsigned char *row = st + box * kBoxBytes + b0 * 128;
-                        const float4 xa = *reinterpret_cast<const float4 *>(row + ((j0 ^ sw) << 4));
-                        const float4 xb =
-                            *reinterpret_cast<const float4 *>(row + (((j0 + 1) ^ sw) << 4));
-                        uint4 hv, lv;
-                        if (tail)
-                            convert_unit<true>(xa, xb, c, nsc, u, lim, bsum, ymax, hv, lv);
-                        else
-                            convert_unit<false>(xa, xb, c, nsc, u, lim, bsum, ymax, hv, lv);
-                        *reinterpret_cast<uint4 *>(ohi + ((u ^ sw) << 4)) = hv;
-                        *reinterpret_cast<uint4 *>(olo + ((u ^ sw) << 4)) = lv;
-                    }
+                    if (fr.vec)
+                        convert_row<false, kUnits>(row, 0, c, nsc, u0, sw, tail, lim, ohi,
+                                                   ohi + kOpBytes, bsum, ymax);
+                    else
+                        convert_row<true, kUnits>(row, m, c, nsc, u0, sw, tail, lim, ohi,
+                                                  ohi + kOpBytes, bsum, ymax);
                 }
                 asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
                 __syncwarp();
-                if (lane == 0) mbar_arrive(&bars.op_full[t]);
+                if (lane == 0) {
+                    mbar_arrive(&bars.op_full[t]);
+                    mbar_arrive(&bars.empty[slot]);
+                }
                 const int j = ji % G::kSegChunks;
                 if (j == G::kSegChunks - 1 || ji == nch - 1) {
                     drain_segment<kAccHH, kParts, G::kXCol>(tmem, warp, lane, B, Np, 0, 0, j + 1,
@@ -1366,21 +1414,22 @@ gram_tc_items_kernel(const BatchFrame one, const BatchFrame *__restrict__ frames
                     ++s;
                 }
             }
-            if (stop) break;
             // end of the item: flags and band sums
             if (!isfinite(bsum)) atomicOr(&fr.ctl->status, ST_NONFINITE_CUBE);
             if (!(ymax < kFp16Max)) range_item = 1;
             if (part >= 1) bsum_sh[part - 1][b0] = bsum;
-            conv_bar(kConv);
+            // every converter is here, also after a wait gave up
+            if (conv_bar_or(kConv, stop)) {
+                stop = true;
+                break;
+            }
             if (part == 0 && b0 < B) {
                 float t = bsum;
                 for (int q = 1; q < kParts; ++q) t += bsum_sh[q - 1][b0];
                 fr.sum_part[(size_t)item.part * B + b0] = t * isc_sh[b0];
             }
             if (cv == 0 && range_item && l < kMaxLocalItems) flagged[l >> 6] |= 1ull << (l & 63);
-            conv_bar(kConv);  // isc_sh, bsum_sh and range_item are the next item's now
         }
-        asm volatile("cp.async.wait_all;" ::: "memory");
     }
     if (tid == 32 && ncommit > 0) {
         for (uint32_t k = 0; k < kWaitLimit; ++k)
@@ -1453,8 +1502,6 @@ bool gram_tc_usable(const float *cube, int B, long N)
            (reinterpret_cast<uintptr_t>(cube) & 3u) == 0;
 }
 
-size_t gram_tc_smem_bytes() { return Cfg<>::kSmem; }
-
 // One tensor-core CTA per SM at most, each on a contiguous chunk range of
 // `per` chunks; the last partial may hold fewer.
 long gram_tc_per(long N, int n_part, int sm_count)
@@ -1512,10 +1559,10 @@ template <int kSt>
 void launch_items(const BatchFrame &one, const BatchFrame *frames, const GramItem *items,
                   const int *cta_items, int n_items, int B, int grid, cudaStream_t st)
 {
-    const size_t smem = Cfg<kSt>::kSmem;
+    const size_t smem = kItemSmem<kSt>;
     cudaFuncSetAttribute(gram_tc_items_kernel<kSt>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                          (int)smem);
-    launch_pdl(gram_tc_items_kernel<kSt>, dim3(grid), dim3(Cfg<kSt>::kThreads), smem, st, one, frames,
+    launch_pdl(gram_tc_items_kernel<kSt>, dim3(grid), dim3(kItemThreads<kSt>), smem, st, one, frames,
                items, cta_items, n_items, B);
 }
 }  // namespace
