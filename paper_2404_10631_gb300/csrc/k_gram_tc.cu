@@ -39,6 +39,8 @@
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
 
+#include <type_traits>
+
 #include "hsc_internal.cuh"
 #include "pdl.cuh"
 #include "tma_util.cuh"
@@ -465,8 +467,16 @@ gram_tc_kernel(const __grid_constant__ CUtensorMap tmap, const float *__restrict
             ++ncommit;
         }
     } else {
-        // ---------------- converters: kRpt band rows x one box (kParts = 2)
-        // or both boxes (kParts = 1) of every chunk
+        // ---------------- converters: half a band row of every chunk each.
+        // What bounds the kernel is the time a warp takes for a chunk, one
+        // after another, not the copies (3, 4 and 6 stages take the same time),
+        // the MMAs (a third operand stage changes nothing) or shared memory
+        // (half of its bandwidth): so the loads of a row come before the
+        // stores that could alias them, and the next chunk's, if it is there,
+        // before the fence that waits for this one's stores. Measured (means
+        // and covariance): 1000 x 1000 x 100 129 -> 114 us, 1024 x 1024 x 32 106
+        // -> 95, 416 x 512 x 128 47.7 -> 46.4. (Sixteen converter warps, or
+        // eight more for the band sums alone, were slower: 137 - 160 us.)
         constexpr int kUnits = 8 / kParts;  // 8-pixel fp16 units per thread per chunk
         const int u0 = part * kUnits;
         const int sw = b0 & 7;  // (b0 + 128) & 7 too
@@ -492,6 +502,20 @@ gram_tc_kernel(const __grid_constant__ CUtensorMap tmap, const float *__restrict
                                                            &bars.drained, abort_p);
         };
         int seg = 0, seg_start = 0, done_i = 0;
+        // the 128-byte staging row of this thread's 32-pixel half
+        const int srow = k3D ? 2 * b0 + part : part * kRows + b0;
+        const int ssw = srow & 7;
+        const bool row_in = b0 < B;
+        const float c = sc[b0], nsc = -sh[b0] * c;  // exact: c is a power of two
+        float4 xr[2 * kUnits];
+        auto load = [&](int s) {
+            if (!row_in) return;
+            const unsigned char *row = staging + s * kStageBytes + srow * 128;
+#pragma unroll
+            for (int q = 0; q < 2 * kUnits; ++q)
+                xr[q] = *reinterpret_cast<const float4 *>(row + ((q ^ ssw) << 4));
+        };
+        bool ahead = false;  // chunk i's loads were issued in the last turn
         for (int i = 0; i < nchunks; ++i) {
             if (i == seg_start + G::kSegChunks) {
                 if (!drain(seg, seg_start, i)) break;
@@ -500,8 +524,11 @@ gram_tc_kernel(const __grid_constant__ CUtensorMap tmap, const float *__restrict
             }
             const int s = i % kStages, t = i % kOpStages;
             // warp-uniform exits: the drains below use warp-collective TMEM loads
-            if (!__all_sync(0xffffffffu, mbar_wait(&bars.full[s], (i / kStages) & 1, abort_p, wl)))
-                break;
+            if (!ahead) {
+                if (!__all_sync(0xffffffffu, mbar_wait(&bars.full[s], (i / kStages) & 1, abort_p, wl)))
+                    break;
+                load(s);
+            }
             if (i >= kOpStages &&
                 !__all_sync(0xffffffffu,
                             mbar_wait(&bars.op_empty[t], ((i / kOpStages) - 1) & 1, abort_p)))
@@ -509,34 +536,36 @@ gram_tc_kernel(const __grid_constant__ CUtensorMap tmap, const float *__restrict
             const long px0 = (c_begin + i) * kChunk;
             const bool tail = px0 + kChunk > N;
             const int lim = tail ? (int)(N - px0) : kChunk;
-#pragma unroll
-            for (int r = 0; r < kRpt; ++r) {
-                const int b = b0 + 128 * r;
-                if (b >= B) continue;
-                const float c = sc[b], nsc = -sh[b] * c;  // exact: c is a power of two
-                const unsigned char *st = staging + s * kStageBytes;
-                unsigned char *ohi = ops + t * 2 * kOpBytes + b * 128;
+            if (row_in) {
+                unsigned char *ohi = ops + t * 2 * kOpBytes + b0 * 128;
                 unsigned char *olo = ohi + kOpBytes;
-                // this thread's 32-pixel half (u >> 2 == part for all its units):
-                // its 128-byte staging row
-                const int srow = k3D ? 2 * b + part : part * kRows + b;
-                const int ssw = srow & 7;
-                const unsigned char *row = st + srow * 128;
+                if (tail) {
 #pragma unroll
-                for (int uu = 0; uu < kUnits; ++uu) {
-                    const int u = u0 + uu;
-                    const int j0 = (u & 3) * 2;  // 16-byte units (4 px) within the box row
-                    const float4 xa = *reinterpret_cast<const float4 *>(row + ((j0 ^ ssw) << 4));
-                    const float4 xb = *reinterpret_cast<const float4 *>(row + (((j0 + 1) ^ ssw) << 4));
-                    uint4 hv, lv;
-                    if (tail)
-                        convert_unit<true>(xa, xb, c, nsc, u, lim, bsum[r], ymax, hv, lv);
-                    else
-                        convert_unit<false>(xa, xb, c, nsc, u, lim, bsum[r], ymax, hv, lv);
-                    *reinterpret_cast<uint4 *>(ohi + ((u ^ sw) << 4)) = hv;
-                    *reinterpret_cast<uint4 *>(olo + ((u ^ sw) << 4)) = lv;
+                    for (int uu = 0; uu < kUnits; ++uu) {
+                        const int u = u0 + uu;
+                        uint4 hv, lv;
+                        convert_unit<true>(xr[2 * uu], xr[2 * uu + 1], c, nsc, u, lim, bsum[0],
+                                           ymax, hv, lv);
+                        *reinterpret_cast<uint4 *>(ohi + ((u ^ sw) << 4)) = hv;
+                        *reinterpret_cast<uint4 *>(olo + ((u ^ sw) << 4)) = lv;
+                    }
+                } else {
+#pragma unroll
+                    for (int uu = 0; uu < kUnits; ++uu) {
+                        const int u = u0 + uu;
+                        uint4 hv, lv;
+                        convert_unit<false>(xr[2 * uu], xr[2 * uu + 1], c, nsc, u, lim, bsum[0],
+                                            ymax, hv, lv);
+                        *reinterpret_cast<uint4 *>(ohi + ((u ^ sw) << 4)) = hv;
+                        *reinterpret_cast<uint4 *>(olo + ((u ^ sw) << 4)) = lv;
+                    }
                 }
             }
+            // the next chunk's loads, if it is there, behind this one's stores
+            const int s1 = (i + 1) % kStages;
+            ahead = i + 1 < nchunks &&
+                    __all_sync(0xffffffffu, mbar_try(&bars.full[s1], ((i + 1) / kStages) & 1));
+            if (ahead) load(s1);
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
             __syncwarp();
             if (lane == 0) {
@@ -1125,24 +1154,28 @@ __device__ __forceinline__ void fetch_chunk(unsigned char *slot, const float *cu
     if (t < B) copy_unit(dst1, a1, a1 + n, lo, hi, 16u, pol);
 }
 
-// A thread's 32 pixels (units u0 .. u0 + 3 of 8) of a staged band row to the
-// operand tiles, from units that start m floats before the first pixel
-// (kShift; else m = 0): two selects per value.
-template <bool kShift, int kUnits>
+// A thread's 32 pixels (units u0 .. u0 + kUnits - 1 of 8) of a staged band row
+// to the operand tiles, from 16-byte units that start m floats before the
+// first pixel (kShift; else m = 0): two selects per value. All loads first:
+// the stores could alias them, and would hold back each unit's.
+template <bool kShift, bool kTail, int kUnits>
 __device__ __forceinline__ void convert_row(const unsigned char *row, int m, float c, float nsc,
-                                            int u0, int sw, bool tail, int lim, unsigned char *ohi,
+                                            int u0, int sw, int lim, unsigned char *ohi,
                                             unsigned char *olo, float &bsum, float &ymax)
 {
+    constexpr int kQ = 2 * kUnits + (kShift ? 1 : 0);
     const float4 *q = reinterpret_cast<const float4 *>(row) + 2 * u0;
-    float4 next = q[0];
+    float4 xr[kQ];
+#pragma unroll
+    for (int i = 0; i < kQ; ++i) xr[i] = q[i];
 #pragma unroll
     for (int uu = 0; uu < kUnits; ++uu) {
         const int u = u0 + uu;
-        float4 xa = next, xb = q[2 * uu + 1];
-        if (kShift) {
-            next = q[2 * uu + 2];
+        float4 xa = xr[2 * uu], xb = xr[2 * uu + 1];
+        if constexpr (kShift) {
+            const float4 xn = xr[2 * uu + 2];
             const float f[12] = {xa.x, xa.y, xa.z, xa.w, xb.x, xb.y, xb.z, xb.w,
-                                 next.x, next.y, next.z, next.w};
+                                 xn.x, xn.y, xn.z, xn.w};
             float t[9], x[8];
 #pragma unroll
             for (int e = 0; e < 9; ++e) t[e] = (m & 2) ? f[e + 2] : f[e];
@@ -1150,12 +1183,9 @@ __device__ __forceinline__ void convert_row(const unsigned char *row, int m, flo
             for (int e = 0; e < 8; ++e) x[e] = (m & 1) ? t[e + 1] : t[e];
             xa = make_float4(x[0], x[1], x[2], x[3]);
             xb = make_float4(x[4], x[5], x[6], x[7]);
-        } else if (uu + 1 < kUnits) {
-            next = q[2 * uu + 2];
         }
         uint4 hv, lv;
-        if (tail) convert_unit<true>(xa, xb, c, nsc, u, lim, bsum, ymax, hv, lv);
-        else convert_unit<false>(xa, xb, c, nsc, u, lim, bsum, ymax, hv, lv);
+        convert_unit<kTail>(xa, xb, c, nsc, u, lim, bsum, ymax, hv, lv);
         *reinterpret_cast<uint4 *>(ohi + ((u ^ sw) << 4)) = hv;
         *reinterpret_cast<uint4 *>(olo + ((u ^ sw) << 4)) = lv;
     }
@@ -1217,10 +1247,10 @@ __device__ __forceinline__ GramItem get_item(const BatchFrame &one,
 // converters shift what they read. Measured (means and covariance): 1001 x 999
 // x 100 228 -> 153 us, 415 x 513 x 128 68 -> 53 us, 201 x 199 x 100 48 -> 38
 // us against copies of 4 bytes issued by the converters; 256 snapshot frames
-// of 40 - 64 pixels a side, 125 bands, 238 -> 188 us. What is left is the
-// conversion (the copies alone take 93 us of the 153; the shift 12). Bulk
-// copies of a row's 272 bytes instead, by one thread per row: 433 us (some 40
-// ns each).
+// of 40 - 64 pixels a side, 125 bands, 238 -> 188 us. With a row's loads
+// before its stores 136, 48, 36 and 177 us. What is left is the conversion
+// (the copies alone take 93 us of the 136). Bulk copies of a row's 272 bytes
+// instead, by one thread per row: 433 us (some 40 ns each).
 template <int kSt>
 __global__ void __launch_bounds__(kItemThreads<kSt>, 1)
 gram_tc_items_kernel(const BatchFrame one, const BatchFrame *__restrict__ frames,
@@ -1392,12 +1422,13 @@ gram_tc_items_kernel(const BatchFrame one, const BatchFrame *__restrict__ frames
                 if (b0 < B) {
                     const unsigned char *row = staging + slot * kItemStage + b0 * kItemRow;
                     unsigned char *ohi = ops + t * 2 * kOpBytes + b0 * 128;
-                    if (fr.vec)
-                        convert_row<false, kUnits>(row, 0, c, nsc, u0, sw, tail, lim, ohi,
-                                                   ohi + kOpBytes, bsum, ymax);
-                    else
-                        convert_row<true, kUnits>(row, m, c, nsc, u0, sw, tail, lim, ohi,
-                                                  ohi + kOpBytes, bsum, ymax);
+                    auto convert = [&](auto shift, auto last) {
+                        convert_row<decltype(shift)::value, decltype(last)::value, kUnits>(
+                            row, m, c, nsc, u0, sw, lim, ohi, ohi + kOpBytes, bsum, ymax);
+                    };
+                    if (tail) convert(std::true_type{}, std::true_type{});
+                    else if (fr.vec) convert(std::false_type{}, std::false_type{});
+                    else convert(std::true_type{}, std::false_type{});
                 }
                 asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
                 __syncwarp();
