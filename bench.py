@@ -150,7 +150,7 @@ def stage_work(f, knn_pairs_per_launch=None):
     it: HBM bytes for the two passes over the cube and the normalisation,
     FP32-pipe lane-ops for the KNN (4 per (pixel, candidate) pair it
     evaluates: the whole window for the full scan, the measured count for the
-    pruned walk), and no roofline for the one-CTA eigensolver (a latency,
+    pruned search), and no roofline for the eigensolver (a latency,
     reported in microseconds). The covariance also carries its tensor work
     (2 B^2 flops per pixel)."""
     B, H, W = f.cube.shape
@@ -537,8 +537,8 @@ def frame_stream(hsc, f, dev, args, world, F, fp32_rate, fp32_peak_note, with_e2
                               "evaluated; peak: " + fp32_peak_note)
         else:
             entry["us_per_launch"] = 1e3 * ms
-            entry["note"] = ("a latency, no roofline: one CTA per frame up to 128 bands; for "
-                             "129-256 bands the first sweep on a 16-CTA cluster, then one CTA; "
+            entry["note"] = ("a latency, no roofline: one CTA per frame up to 128 bands, a "
+                             "cluster of 8 for 129-256; "
                              "with frames in flight the other frames' GPU-wide stages run "
                              "beside it")
         if name == "moments":

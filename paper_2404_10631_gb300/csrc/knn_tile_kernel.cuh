@@ -25,9 +25,8 @@
 //
 // Measured, walk and second pass together, against one pixel per lane with
 // every candidate of the disk keyed and P gathered by dependent loads:
-// 416 x 512, K = 40, 14 rows, lambda 1, 4 classes: 66 -> 29 us; 1024 x 1024:
-// 183 -> 40 us; 509 x 401, K = 24, 9 rows, lambda 0.5, 3 classes: 275 -> 68 us;
-// 416 x 512 with a window of 5 rows, which cuts the disk of K = 40: 85 -> 55 us.
+// 416 x 512, K = 40, 14 rows, lambda 1, 4 classes: 66 -> 23 us; 1024 x 1024:
+// 183 -> 39 us; 509 x 401, K = 24, 9 rows, lambda 0.5, 3 classes: 275 -> 36 us.
 //
 // What bounds it: instruction issue (1024 x 1024: 50% of the slots, L1 at 72%)
 // and, on frames of a few hundred thousand
