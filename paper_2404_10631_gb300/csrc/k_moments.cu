@@ -17,7 +17,7 @@
 namespace hsc {
 namespace {
 
-constexpr int kGramThreads = 256;
+constexpr int kGramThreads = 288;
 constexpr int kGramChunk = 32;   // pixels staged per step
 constexpr int kTile = 8;         // 8x8 accumulator tile per thread
 
@@ -226,23 +226,45 @@ __device__ __forceinline__ dfl cov_entry(float g, float gl, dfl inv, dfl db, dfl
     return df_add(df_mul({g, gl}, inv), {-q.h, -q.l});
 }
 
-// grid.x = pixel partitions, grid.y = groups of 256 output tiles (B > 128).
-// Shared: Yt[kGramChunk][Bp + 4] (pixel-major, shifted values).
-__global__ void __launch_bounds__(kGramThreads)
-gram_partial_kernel(const float *__restrict__ cube, int B, int Bp, long N,
+// Covariance on the FP32 pipe: frames the tensor-core forms do not take (129 -
+// 256 bands with N % 32 != 0, more than 256 bands) and HSC_COV_FP32_PIPE.
+// grid.x = pixel partitions, grid.y = groups of per_cta of the tiles (ti, tj),
+// tj <= ti, of 8 x 8 entries: the half the reduction reads. A thread holds a
+// tile's 64 sums and takes the pixels one after another.
+// Shared: Yt[kGramChunk][Bp + 4], pixel-major shifted values, a pixel's bands
+// in two planes (b % 8 < 4 and >= 4), so that the lanes of a warp, which share
+// ti and have consecutive tj, read consecutive 16-byte units; Bp / 4 + 1 is
+// odd, so the lanes of a staging store (one pixel each) fall into different
+// banks too. kAhead (up to 256 bands): the next chunk's values are loaded into
+// registers before this one's sums; above, loaded and stored in turn.
+// Measured (means and covariance): 1023 x 1024 x 256 10.3 -> 4.8 ms, 333 x 500 x
+// 224 1.51 -> 0.76 ms, 60 x 60 x 256 301 -> 230 us, 40 x 41 x 129 205 -> 141 us,
+// against 256 tiles per CTA of the whole square, loaded and stored in turn
+// with 4-way bank conflicts. The FMAs are a third of the issue slots: what is
+// left is the wait for the loads (nine warps per SM) and, with few
+// partitions, the last round of CTAs.
+template <bool kAhead>
+__global__ void __launch_bounds__(kGramThreads, 1)
+gram_partial_kernel(const float *__restrict__ cube, int B, int Bp, long N, int per_cta,
                     const float *__restrict__ shift, float *__restrict__ gram_part,
                     float *__restrict__ sum_part, Control *ctl)
 {
-    extern __shared__ float smem[];
+    extern __shared__ __align__(16) float smem[];
     pdl_wait();
-    const int ld = Bp + 4;
+    const int ld = Bp + 4, half = Bp / 2;
     float *Yt = smem;                                 // kGramChunk x ld
     float *sh = smem + kGramChunk * ld;               // Bp
     const int tid = threadIdx.x;
     const int nt = Bp / kTile;                        // tiles per side
-    const int tile = blockIdx.y * kGramThreads + tid;
-    const bool has_tile = tile < nt * nt;
-    const int ti = has_tile ? tile / nt : 0, tj = has_tile ? tile % nt : 0;
+    const int tile = blockIdx.y * per_cta + tid;
+    const bool has_tile = tid < per_cta && tile < nt * (nt + 1) / 2;
+    int ti = 0;
+    if (has_tile) {
+        ti = (int)((sqrtf(8.f * (float)tile + 1.f) - 1.f) * 0.5f);
+        while (ti * (ti + 1) / 2 > tile) --ti;
+        while ((ti + 1) * (ti + 2) / 2 <= tile) ++ti;
+    }
+    const int tj = has_tile ? tile - ti * (ti + 1) / 2 : 0;
     const bool do_sums = (blockIdx.y == 0);
 
     for (int b = tid; b < Bp; b += kGramThreads) sh[b] = (b < B) ? shift[b] : 0.f;
@@ -256,36 +278,78 @@ gram_partial_kernel(const float *__restrict__ cube, int B, int Bp, long N,
     for (int a = 0; a < kTile; ++a)
 #pragma unroll
         for (int c = 0; c < kTile; ++c) acc[a][c] = 0.f;
-    float bsum = 0.f;  // thread tid < Bp: running sum of band tid
+    // running sums of the bands tid + kGramThreads q
+    constexpr int kSums = kAhead ? 1 : (1024 + kGramThreads - 1) / kGramThreads;
+    float bsum[kSums];
+#pragma unroll
+    for (int q = 0; q < kSums; ++q) bsum[q] = 0.f;
     bool bad = false;
+    const float *ra = Yt + ti * 4, *rb = Yt + tj * 4;
+
+    // staging: a lane per pixel, four bands of it per store; quad j of a warp
+    constexpr int kWarps = kGramThreads / 32;
+    constexpr int kQuads = (256 / 4 + kWarps - 1) / kWarps;
+    const int warp = tid >> 5, lane = tid & 31;
+    auto load = [&](float (&x)[4], int q, long p) {
+#pragma unroll
+        for (int e = 0; e < 4; ++e)
+            x[e] = 4 * q + e < B && p < p1 ? cube[(size_t)(4 * q + e) * (size_t)N + p] : 0.f;
+    };
+    auto store = [&](const float (&x)[4], int q, long p) {
+        float y[4];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            const bool in = 4 * q + e < B && p < p1;
+            bad |= in && !isfinite(x[e]);
+            y[e] = in ? x[e] - sh[4 * q + e] : 0.f;
+        }
+        *reinterpret_cast<float4 *>(Yt + lane * ld + (q & 1) * half + (q >> 1) * 4) =
+            make_float4(y[0], y[1], y[2], y[3]);
+    };
+    float x[kQuads][4];
+    auto load_all = [&](long pc) {
+#pragma unroll
+        for (int j = 0; j < kQuads; ++j)
+            if (warp + kWarps * j < Bp / 4) load(x[j], warp + kWarps * j, pc + lane);
+    };
+    if (kAhead) load_all(p0);
 
     for (long pc = p0; pc < p1; pc += kGramChunk) {
         __syncthreads();
-        for (int idx = tid; idx < Bp * kGramChunk; idx += kGramThreads) {
-            int b = idx / kGramChunk, pp = idx % kGramChunk;
-            long p = pc + pp;
-            float y = 0.f;
-            if (b < B && p < p1) {
-                float x = cube[(size_t)b * (size_t)N + p];
-                bad |= !isfinite(x);
-                y = x - sh[b];
+        if (kAhead) {
+#pragma unroll
+            for (int j = 0; j < kQuads; ++j)
+                if (warp + kWarps * j < Bp / 4) store(x[j], warp + kWarps * j, pc + lane);
+        } else {
+            for (int q = warp; q < Bp / 4; q += kWarps) {
+                load(x[0], q, pc + lane);
+                store(x[0], q, pc + lane);
             }
-            Yt[pp * ld + b] = y;
         }
         __syncthreads();
-        if (do_sums && tid < Bp) {
-            float s = 0.f;
-            for (int pp = 0; pp < kGramChunk; ++pp) s += Yt[pp * ld + tid];
-            bsum += s;
+        if (kAhead && pc + kGramChunk < p1) load_all(pc + kGramChunk);
+        if (do_sums) {
+#pragma unroll
+            for (int q = 0; q < kSums; ++q) {
+                const int b = tid + kGramThreads * q;
+                if (b < Bp) {
+                    const float *col = Yt + ((b >> 2) & 1) * half + (b >> 3) * 4 + (b & 3);
+                    float t = 0.f;
+#pragma unroll 8
+                    for (int pp = 0; pp < kGramChunk; ++pp) t += col[pp * ld];
+                    bsum[q] += t;
+                }
+            }
         }
         if (has_tile) {
 #pragma unroll 4
             for (int pp = 0; pp < kGramChunk; ++pp) {
-                const float4 *ra = reinterpret_cast<const float4 *>(Yt + pp * ld + ti * kTile);
-                const float4 *rb = reinterpret_cast<const float4 *>(Yt + pp * ld + tj * kTile);
-                float4 a0 = ra[0], a1 = ra[1], b0 = rb[0], b1 = rb[1];
-                float av[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
-                float bv[8] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
+                const float4 a0 = *reinterpret_cast<const float4 *>(ra + pp * ld);
+                const float4 a1 = *reinterpret_cast<const float4 *>(ra + pp * ld + half);
+                const float4 b0 = *reinterpret_cast<const float4 *>(rb + pp * ld);
+                const float4 b1 = *reinterpret_cast<const float4 *>(rb + pp * ld + half);
+                const float av[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
+                const float bv[8] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
 #pragma unroll
                 for (int a = 0; a < kTile; ++a)
 #pragma unroll
@@ -308,14 +372,19 @@ gram_partial_kernel(const float *__restrict__ cube, int B, int Bp, long N,
             }
         }
     }
-    if (do_sums && tid < B) sum_part[(size_t)blockIdx.x * B + tid] = bsum;
+    if (do_sums) {
+#pragma unroll
+        for (int q = 0; q < kSums; ++q) {
+            const int b = tid + kGramThreads * q;
+            if (b < B) sum_part[(size_t)blockIdx.x * B + b] = bsum[q];
+        }
+    }
 }
 
 // C_bc = (sum_i G_i[b][c]) / N - delta_b delta_c for b <= c, mirrored, in
 // FP64 and as FP32 (hi, lo) pairs, and mu_b = s_b + delta_b with delta_b =
 // (1/N) sum_i S_i[b] (S_i the partial sums of y). Each partial holds entry
-// (b, c) at c * B + b (the tensor-core Gram writes that half of its block;
-// the FP32 version writes the whole symmetric matrix). A CTA takes 32
+// (b, c) at c * B + b (only that half is written). A CTA takes 32
 // consecutive positions e = c*B + b; its 8 warps each sum every 8th partial
 // of G, and of S for the entry's two bands, in double-float with eight loads
 // of each issued ahead of the additions (coalesced across the 32 positions); then the
@@ -521,14 +590,16 @@ cudaError_t launch_moments(const float *cube, int B, long N, const PcaScratch &s
     }
     const int Bp = (B + kTile - 1) / kTile * kTile;
     const int nt = Bp / kTile;
-    const int groups = (nt * nt + kGramThreads - 1) / kGramThreads;
+    const int tiles = nt * (nt + 1) / 2;
+    const int groups = (tiles + kGramThreads - 1) / kGramThreads;
+    const int per_cta = (tiles + groups - 1) / groups;
     size_t smem = sizeof(float) * ((size_t)kGramChunk * (Bp + 4) + Bp);
+    auto kern = Bp <= 256 ? gram_partial_kernel<true> : gram_partial_kernel<false>;
     if (smem > 48 * 1024)
-        cudaFuncSetAttribute(gram_partial_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)smem);
+        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     dim3 grid(s.n_part, groups);
     const cudaError_t ge =
-        launch_pdl(gram_partial_kernel, grid, dim3(kGramThreads), smem, st, cube, B, Bp, N, s.shift,
+        launch_pdl(kern, grid, dim3(kGramThreads), smem, st, cube, B, Bp, N, per_cta, s.shift,
                    s.gram_part, s.sum_part, s.ctl);
     if (ge != cudaSuccess) return ge;
     return launch_reductions(B, N, s.n_part, s, st);
