@@ -35,9 +35,11 @@ constexpr int kFrameThreads = 128;
 // KC = 0: projection only. PX = pixels per thread (4, with 16-byte loads
 // when kVec, or 1).
 // kF64: the coupling to FP64-level accuracy (a kernel of its own: the refined
-// solve is several times the code of the plain one).
+// solve is several times the code of the plain one). From five classes on it
+// is held to 128 registers, four CTAs of 128 threads per SM: 415 x 513 x 128, 7
+// classes 95 -> 71 us, 8 classes 119 -> 97 us.
 template <int KC, int PX, bool kVec, bool kF64>
-__global__ void __launch_bounds__(kThreads)
+__global__ void __launch_bounds__(kThreads, kF64 && KC >= 5 && PX == 1 ? 2 : 0)
 project_svm_kernel(const float *__restrict__ cube, int B, long N,
                    const float *__restrict__ v1f, const float *__restrict__ muf,
                    const float *__restrict__ w, const float *__restrict__ bias,
@@ -64,9 +66,11 @@ project_svm_kernel(const float *__restrict__ cube, int B, long N,
 
 // Stage-major batch: CTA i takes work item i (one frame's groups of 4
 // pixels, 16-byte loads where the frame allows them); labels are not
-// written (the KNN gives them).
+// written (the KNN gives them). Three CTAs per SM, two where the refined
+// coupling of five and more classes would spill (256 snapshot frames, 6
+// classes, the call: 897 -> 596 us).
 template <int KC, bool kF64>
-__global__ void __launch_bounds__(kThreads, 3)
+__global__ void __launch_bounds__(kThreads, kF64 && KC >= 5 ? 2 : 3)
 project_svm_batch_kernel(const BatchFrame *__restrict__ frames, const PixItem *__restrict__ items,
                          int B, const float *__restrict__ w, const float *__restrict__ bias,
                          const float *__restrict__ pa, const float *__restrict__ pb)
@@ -182,8 +186,10 @@ cudaError_t launch_project_svm(const float *cube, int B, long N, const float *v1
     // classes 17.2 / 13.2 / 13.1; 48 x 48 x 125, 4 classes 16.0 / 12.1 / 10.4.
     if (px == 0) px = N < 65536 || k >= 6 ? 1 : 4;
     if (px == 4 && (k == 2 || k == 3 || k == 5)) px = 2;
-    // the refined coupling solves: one or two pixels (its code and registers)
-    if (couple_f64 && k > 0 && px == 4) px = 2;
+    // the refined coupling solves, by their code and registers: two pixels at
+    // most, one from five classes on (415 x 513 x 128, two / one: 4 classes 31 /
+    // 38 us, 5 classes 50 / 42, 6 classes 64 / 57, 8 classes 141 / 97)
+    if (couple_f64 && k > 0) px = k >= 5 ? 1 : (px == 4 ? 2 : px);
 #define HSC_SVM_PX(PX, VEC, F64)                                                                   \
     dispatch_k<PX, VEC, F64>(k, cube, B, N, v1f, muf, I_raw, model, probs, svm_labels, ctl,        \
                              sm_count, st, max_blocks, P4)

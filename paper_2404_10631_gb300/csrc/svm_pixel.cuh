@@ -27,15 +27,22 @@ __host__ __device__ constexpr int svm_stride(int k)
 }
 
 // The coupling of one pixel: (Q + e e^T) y = e, p = y / sum y, by LDL^T in
-// FP32. kRefine (HSC_SVM_COUPLE_F64): one step of iterative refinement to
-// FP64-level accuracy, in double-float on the FP32 pipe: the residual
-// e - (Q + e e^T) y with the matrix's entries as FP32 pairs (1 - r is exact as
-// one, the products are split by an FMA), one more solve with the FP32
-// factors, and sum and quotient in pairs. The matrix's condition number is
-// below 25, so the FP32 solution is good to 1e-6 and the corrected one to
-// 1e-12 before it is rounded to FP32. (In FP64 arithmetic throughout, 250
-// operations and 7 divisions for 6 classes at under two per clock and SM:
-// 509 x 401 x 100, 6 classes 112 us, this way 49 us.)
+// FP32. kRefine (HSC_SVM_COUPLE_F64): two steps of iterative refinement to
+// better than FP64's accuracy, in double-float on the FP32 pipe. Solved is Q y
+// = c e, c = 1 - e^T y kept as an unknown of its own: in c - (Q y)_i the terms
+// of a class that loses every pair are all as small as its y_i, where 1 -
+// ((Q + e e^T) y)_i would cancel against the winner's y = 1 and lose them (one
+// correction in that form: relative errors up to 1e-6 for p = 1e-8). The
+// products r_ij r_ji and squares r_ji^2 are FP32 pairs (1 - r is exact as one,
+// products are split by an FMA), the correction d comes from the FP32 factors
+// of Q + e e^T (condition number below 25: each step gains six digits), then
+// y += d and c -= e^T d as pairs; sum and quotient in pairs. Against exact
+// rational arithmetic (consistent, cyclic and clipped r, 2 to 8 classes) p is
+// the correctly rounded FP32 value in 99.5% of the cases, the FP64 LDL^T's in
+// 99.3%, and never more than 1.00 half-units off.
+// 509 x 401 x 100, 6 classes: 46 us with one correction, 47 us with these two,
+// 112 us in FP64 arithmetic throughout (250 operations and 7 divisions at under
+// two per clock and SM).
 template <int KC, bool kRefine>
 __device__ __forceinline__ void couple_solve(const float *r /* M, pair order */, float *p)
 {
@@ -108,20 +115,11 @@ __device__ __forceinline__ void couple_solve(const float *r /* M, pair order */,
 #pragma unroll
         for (int i = 0; i < KC; ++i) p[i] = y[i] * inv;
     } else {
-        // res_i = 1 - sum_j A_ij y_j and the diagonal entries, as pairs
-        float rs[KC], rl[KC], ds[KC], dl[KC];
+        // Q's entries as pairs: r_ij r_ji per class pair, sum_j r_ji^2 per class
+        constexpr int M = KC * (KC - 1) / 2;
+        float qh[M], ql[M], ds[KC], dl[KC];
 #pragma unroll
-        for (int i = 0; i < KC; ++i) {
-            rs[i] = ds[i] = 1.f;
-            rl[i] = dl[i] = 0.f;
-        }
-        auto sub = [&](int i, float ah, float al, float yj) {  // res_i -= (ah + al) yj
-            const float q = __fmul_rn(ah, yj);
-            const float qe = __fmaf_rn(ah, yj, -q);
-            float e;
-            two_sum(rs[i], -q, rs[i], e);
-            rl[i] = __fadd_rn(rl[i], __fsub_rn(e, __fmaf_rn(al, yj, qe)));
-        };
+        for (int i = 0; i < KC; ++i) ds[i] = dl[i] = 0.f;
         auto add_sq = [&](int i, float h, float l) {  // diagonal i += (h + l)^2
             const float q = __fmul_rn(h, h);
             const float qe = __fmaf_rn(__fmul_rn(2.f, h), l, __fmaf_rn(h, h, -q));
@@ -129,47 +127,90 @@ __device__ __forceinline__ void couple_solve(const float *r /* M, pair order */,
             two_sum(ds[i], q, ds[i], e);
             dl[i] = __fadd_rn(dl[i], __fadd_rn(e, qe));
         };
-        int m = 0;
+        {
+            int m = 0;
 #pragma unroll
-        for (int i = 0; i < KC; ++i)
+            for (int i = 0; i < KC; ++i)
 #pragma unroll
-            for (int j = i + 1; j < KC; ++j, ++m) {
-                float h, l;  // 1 - r_ij = r_ji
-                two_sum(1.f, -r[m], h, l);
-                add_sq(i, h, l);
-                add_sq(j, r[m], 0.f);
-                const float q = __fmul_rn(r[m], h);
-                const float qe = __fmaf_rn(r[m], l, __fmaf_rn(r[m], h, -q));
-                float ah, al;
-                two_sum(1.f, -q, ah, al);
-                al = __fsub_rn(al, qe);
-                sub(i, ah, al, y[j]);
-                sub(j, ah, al, y[i]);
-            }
-        float d[KC];
+                for (int j = i + 1; j < KC; ++j, ++m) {
+                    float h, l;  // 1 - r_ij = r_ji
+                    two_sum(1.f, -r[m], h, l);
+                    add_sq(i, h, l);
+                    add_sq(j, r[m], 0.f);
+                    qh[m] = __fmul_rn(r[m], h);
+                    ql[m] = __fmaf_rn(r[m], l, __fmaf_rn(r[m], h, -qh[m]));
+                }
+        }
+        float yl[KC], ch = 1.f, cl = 0.f;  // y = y + yl, c = ch + cl
 #pragma unroll
         for (int i = 0; i < KC; ++i) {
             const dfl a = fast_two_sum(ds[i], dl[i]);
-            sub(i, a.h, a.l, y[i]);
-            d[i] = __fadd_rn(rs[i], rl[i]);
+            ds[i] = a.h;
+            dl[i] = a.l;
+            yl[i] = 0.f;
+            ch -= y[i];
         }
-        solve(d);
+#pragma unroll 1
+        for (int it = 0; it < 2; ++it) {
+            float rs[KC], rl[KC];  // c - (Q y)_i
+#pragma unroll
+            for (int i = 0; i < KC; ++i) {
+                rs[i] = ch;
+                rl[i] = cl;
+            }
+            auto add = [&](int i, float ah, float al, int j) {  // res_i += (ah + al) y_j
+                const float q = __fmul_rn(ah, y[j]);
+                float t = __fmaf_rn(ah, y[j], -q);
+                t = __fmaf_rn(al, y[j], t);
+                t = __fmaf_rn(ah, yl[j], t);
+                float e;
+                two_sum(rs[i], q, rs[i], e);
+                rl[i] = __fadd_rn(rl[i], __fadd_rn(e, t));
+            };
+            int m = 0;
+#pragma unroll
+            for (int i = 0; i < KC; ++i)
+#pragma unroll
+                for (int j = i + 1; j < KC; ++j, ++m) {
+                    add(i, qh[m], ql[m], j);
+                    add(j, qh[m], ql[m], i);
+                }
+            float d[KC], g = 0.f;
+#pragma unroll
+            for (int i = 0; i < KC; ++i) {
+                add(i, -ds[i], -dl[i], i);
+                d[i] = __fadd_rn(rs[i], rl[i]);
+            }
+            solve(d);
+            float e;
+#pragma unroll
+            for (int i = 0; i < KC; ++i) {
+                g += d[i];
+                float t;
+                two_sum(y[i], d[i], t, e);
+                const dfl n = fast_two_sum(t, __fadd_rn(yl[i], e));
+                y[i] = n.h;
+                yl[i] = n.l;
+            }
+            float t;
+            two_sum(ch, -g, t, e);
+            const dfl n = fast_two_sum(t, __fadd_rn(cl, e));
+            ch = n.h;
+            cl = n.l;
+        }
         float s = 0.f, sl = 0.f;
 #pragma unroll
-        for (int i = 0; i < KC; ++i) {  // y + d as a pair (d in its place holds the low part)
-            const dfl t = fast_two_sum(y[i], d[i]);
-            y[i] = t.h;
-            d[i] = t.l;
+        for (int i = 0; i < KC; ++i) {
             float e;
-            two_sum(s, t.h, s, e);
-            sl = __fadd_rn(sl, __fadd_rn(e, t.l));
+            two_sum(s, y[i], s, e);
+            sl = __fadd_rn(sl, __fadd_rn(e, yl[i]));
         }
         const dfl sum = fast_two_sum(s, sl);
         const float inv = 1.f / sum.h;
 #pragma unroll
         for (int i = 0; i < KC; ++i) {
             const float q = __fmul_rn(y[i], inv);
-            const float rem = __fadd_rn(__fmaf_rn(-q, sum.h, y[i]), __fmaf_rn(-q, sum.l, d[i]));
+            const float rem = __fadd_rn(__fmaf_rn(-q, sum.h, y[i]), __fmaf_rn(-q, sum.l, yl[i]));
             p[i] = __fmaf_rn(rem, inv, q);
         }
     }
@@ -248,10 +289,14 @@ __device__ __forceinline__ void finish_svm_pixel(const float (&acc)[KC * (KC - 1
 // Loads in flight per thread in the single-frame launches (kAhead PX registers
 // beside (M + 1) PX accumulators); the batch's kernels, three CTAs of 256
 // threads per SM at 80 registers, take 4.
-constexpr int svm_ahead(int k, int px) { return px == 4 ? 8 : px == 2 ? 16 : (k >= 5 ? 16 : 32); }
+// (24 with the refined coupling of 4 classes: 128 registers, four CTAs per SM.)
+constexpr int svm_ahead(int k, int px, bool f64)
+{
+    return px == 4 ? 8 : px == 2 ? 16 : k >= 5 ? 16 : k == 4 && f64 ? 24 : 32;
+}
 
 template <int KC, int PX, bool kVec, bool kF64, bool kStrided = false,
-          int kAhead = svm_ahead(KC, PX)>
+          int kAhead = svm_ahead(KC, PX, kF64)>
 __device__ __forceinline__ void project_svm_groups(
     const float *__restrict__ cube, int B, long N, const float *ws, const float *sbias,
     const float *sa, const float *sb, bool do_pca, long g_begin, long g_end, long g_step,
