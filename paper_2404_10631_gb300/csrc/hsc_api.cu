@@ -1296,7 +1296,10 @@ hsc_status classify_batch_staged(hsc_ctx *ctx, const hsc_frame *frames, int n_fr
                reinterpret_cast<long long>(model->platt_a),
                reinterpret_cast<long long>(model->platt_b),
                reinterpret_cast<long long>(ctx->stream), reinterpret_cast<long long>(dev),
-               (long long)tab};
+               // offsets and counts baked into the launches: two batches that
+               // agree in all the sums above can differ in these (the sizes of
+               // the second group's frames within one alignment step)
+               (long long)tab, (long long)redo, (long long)claims, n_px};
         if (ctx->sm_exec && sig == ctx->sm_sig) {
             e = cudaGraphLaunch(ctx->sm_exec, ctx->stream);
             if (e != cudaSuccess) return cuda_fail(ctx, e, "cudaGraphLaunch");
