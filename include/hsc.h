@@ -358,7 +358,8 @@ enum {
 hsc_status hsc_profile_enable(hsc_ctx *ctx, int enable);
 /* Diagnostics of the context's last PCA (waits for the stream): FP32 Jacobi
  * sweeps run (the Krylov basis of 129-256 bands counts as one, that of up to
- * 128 as none), FP64 refinement iterations of the leading eigenvector, and the
+ * 128 as none; a frame left to the full kernel adds that one's sweeps), FP64
+ * refinement iterations (corrections and restarts) of the leading eigenvector, and the
  * SM clock cycles spent in each part (cycle pointers nullable). */
 hsc_status hsc_pca_diagnostics(hsc_ctx *ctx, int32_t *sweeps, int32_t *refine_iters,
                                int64_t *sweep_cycles, int64_t *refine_cycles);

@@ -1354,7 +1354,9 @@ if (presweep) {
         for (int ii = tid; ii < B; ii += nthr) muf[ii] = (float)mu[ii];
     if (tid == 0 && !kept) {
         if (!converged) atomicOr(&ctl->status, ST_NOT_CONVERGED);
-        ctl->jacobi_sweeps = (unsigned)sweeps;
+        // (the Krylov basis of 129-256 bands counts as one, left or not)
+        const bool left = flagged && (prm.only_if_flagged || prm.keep_lead);
+        ctl->jacobi_sweeps = (unsigned)sweeps + (left && B > 128 ? 1u : 0u);
         ctl->refine_iters = (unsigned)(refine_iters > kMaxRefine ? kMaxRefine : refine_iters);
         ctl->jacobi_sweep_cycles =
             (unsigned long long)t_sweep + (presweep ? ctl->jacobi_cluster_cycles : 0ull);

@@ -21,8 +21,13 @@
 //     theta_c the mean of the eigenvalues outside the space, from the traces;
 //     until ||r|| <= 1e-13 max(rho, max C_ii) ||v||. On the workloads' frames
 //     two corrections.
-//  4. The sign rule; v / ||v||.
-// A frame this cannot finish (a zero C, no convergence in kMaxRefine steps:
+//  4. Where a correction divides ||r|| by less than 4 (a spectrum that decays
+//     with no floor: what is left of r lies outside the space), the space is
+//     built again, from v and the double-float r; T's leading vector without
+//     its first entry is the next correction, and each restart gains a
+//     Chebyshev polynomial of degree 9 on the gap: 100-fold for a gap of 8%.
+//  5. The sign rule; v / ||v||.
+// A frame this cannot finish (a zero C, two restarts that gained less than 4:
 // a leading eigenvalue hardly separated) is flagged (Control::jac_redo) for
 // the full Jacobi kernel launched behind it.
 //
@@ -42,7 +47,10 @@
 // corrections in one CTA: 87 us; always 10 steps here: 34 us); 1024 x 1024 x 256
 // 29 us (one Jacobi sweep on a 16-CTA cluster, then 10-25 corrections on one
 // CTA: 498 us); 300 x 400 x 200 29 us (450 us, and 3.5 ms for frames whose
-// one-sweep basis did not converge).
+// one-sweep basis did not converge). Eigenvalues e^(-j/8) and e^(-j/12), 200 x
+// 200 pixels: 70 and 84 us with 128 bands, 88 and 126 us with 200 (corrections
+// in the first space only, then the full kernel: 350 and 3200, 1150 and 12500
+// us; the block power basis: 147 and 203, 12200 and 12260 us).
 #include <cuda_runtime.h>
 #include <math.h>
 #include <stdint.h>
@@ -56,8 +64,10 @@ namespace {
 
 constexpr int kThreads = 512;
 constexpr int kSteps = 10;
-constexpr int kMaxRefine = 24;
+constexpr int kMaxRounds = 32;   // restarts at most
+constexpr float kSlow = 16.f;    // a step that divides ||r||^2 by less is slow
 constexpr float kShift = 1e-4f;
+constexpr float kMargin = 4e-6f;
 
 template <int CL>  // CTAs per cluster
 struct Shape {
@@ -154,18 +164,21 @@ __device__ __forceinline__ void store_peer(const void *local, uint32_t rank, flo
     asm volatile("st.shared::cluster.v2.f32 [%0], {%1, %2};" ::"r"(p), "f"(v.x), "f"(v.y) : "memory");
 }
 
-// (x I - T) = L D L^T: f_c = beta_c / D_c and 1 / D_c, the pivots kept above
-// a small positive value (x exceeds T's eigenvalues but for rounding)
+// (x I - T) = L D L^T: f_c = beta_c / D_c and 1 / D_c. x exceeds T's largest
+// eigenvalue by kMargin of it or more, a few dozen FP32 roundings, so every
+// pivot is positive and 1 / D_c at most 1 / (kMargin x). (At the eigenvalue
+// itself a pivot can come out as zero or negative before the last one; kept
+// above 1e-7 x it made the next ones negative too, and their quotients
+// overflowed: three frames of some 1200 were lost so.)
 __device__ __forceinline__ void tri_factor(const float (&al)[kSteps], const float (&be)[kSteps],
                                            float x, float (&f)[kSteps], float (&inv)[kSteps])
 {
-    const float tiny = 1e-7f * x;
-    float d = fmaxf(x - al[0], tiny);
+    float d = x - al[0];
 #pragma unroll
     for (int c = 0; c < kSteps; ++c) {
         inv[c] = __fdividef(1.f, d);
         f[c] = be[c] * inv[c];
-        if (c + 1 < kSteps) d = fmaxf((x - al[c + 1]) - be[c] * f[c], tiny);
+        if (c + 1 < kSteps) d = (x - al[c + 1]) - be[c] * f[c];
     }
 }
 __device__ __forceinline__ void tri_solve(const float (&f)[kSteps], const float (&inv)[kSteps],
@@ -290,233 +303,291 @@ krylov_kernel(int B, EigFrame fr, const BatchFrame *__restrict__ frames)
         else __syncthreads();
     };
 
-    // ---- Lanczos
     const int m = B < kSteps ? B : kSteps;
-    int k = 0;
-    float top = 0.f, prod = 1.f;
+    int k = 0, it = 0, stalled = 0;
+    dfl rho = {0.f, 0.f}, vv = {0.f, 0.f};
+    float e_last = INFINITY, e_round = INFINITY;  // ||r||^2 / ||v||^2 a step and a round ago
+    bool converged = false;
+    long long t1 = 0;
 #pragma unroll 1
-    for (int j = 0;; ++j) {
-        {
-            float a0 = 0.f, a1 = 0.f;
-            const float4 *q = reinterpret_cast<const float4 *>(sm.Q[j] + j0);
+    for (int round = 0;; ++round) {
+        // ---- Lanczos (a restart's first column and its row of T are there)
+        float top = rho.h, prod = 1.f;
+#pragma unroll 1
+        for (int j = round ? 1 : 0;; ++j) {
+            {
+                float a0 = 0.f, a1 = 0.f;
+                const float4 *q = reinterpret_cast<const float4 *>(sm.Q[j] + j0);
 #pragma unroll
-            for (int u = 0; u < kNJ; u += 4) {
-                const float4 v = q[u / 4];
-                a0 = fmaf(ch[u], v.x, a0);
-                a1 = fmaf(ch[u + 1], v.y, a1);
-                a0 = fmaf(ch[u + 2], v.z, a0);
-                a1 = fmaf(ch[u + 3], v.w, a1);
-            }
-            sm.part[sl][rl].x = a0 + a1;
-        }
-        __syncthreads();
-        exchange(false);
-        float *y = sm.y[par];
-        par ^= 1;
-        // two passes: the dot products with the columns so far (warp c) and
-        // the vector's own square (warp j + 1), then the subtraction
-#pragma unroll 1
-        for (int pass = 0; pass < 2; ++pass) {
-            if (warp <= j + 1) {
-                const float d = dot<kPad>(warp <= j ? sm.Q[warp] : y, y, lane);
-                if (lane == 0) {
-                    if (warp <= j) (pass ? sm.cb : sm.ca)[warp] = d;
-                    else sm.n2[pass] = d;
+                for (int u = 0; u < kNJ; u += 4) {
+                    const float4 v = q[u / 4];
+                    a0 = fmaf(ch[u], v.x, a0);
+                    a1 = fmaf(ch[u + 1], v.y, a1);
+                    a0 = fmaf(ch[u + 2], v.z, a0);
+                    a1 = fmaf(ch[u + 3], v.w, a1);
                 }
+                sm.part[sl][rl].x = a0 + a1;
             }
             __syncthreads();
-            if (pass == 0) {
-                if (tid < kPad) {
-                    float v = y[tid];
-#pragma unroll 4
-                    for (int c = 0; c <= j; ++c) v = fmaf(-sm.ca[c], sm.Q[c][tid], v);
-                    y[tid] = v;
+            exchange(false);
+            float *y = sm.y[par];
+            par ^= 1;
+            // two passes: the dot products with the columns so far (warp c) and
+            // the vector's own square (warp j + 1), then the subtraction
+#pragma unroll 1
+            for (int pass = 0; pass < 2; ++pass) {
+                if (warp <= j + 1) {
+                    const float d = dot<kPad>(warp <= j ? sm.Q[warp] : y, y, lane);
+                    if (lane == 0) {
+                        if (warp <= j) (pass ? sm.cb : sm.ca)[warp] = d;
+                        else sm.n2[pass] = d;
+                    }
                 }
                 __syncthreads();
-            }
-        }
-        float b2 = sm.n2[1], v = tid < kPad ? y[tid] : 0.f;
+                if (pass == 0) {
+                    if (tid < kPad) {
+                        float v = y[tid];
 #pragma unroll 4
-        for (int c = 0; c <= j; ++c) {
-            const float d = sm.cb[c];
-            b2 = fmaf(-d, d, b2);
-            if (tid < kPad) v = fmaf(-d, sm.Q[c][tid], v);
-        }
-        // The space is exhausted when what is left of the product is rounding,
-        // and large enough when the product of beta / theta (theta by the
-        // largest alpha so far) is: it bounds the leading Ritz vector's last
-        // component, its share of the residual, up to the gaps.
-        const float alpha = sm.ca[j] + sm.cb[j];
-        top = fmaxf(top, alpha);
-        prod *= fminf(1.f, b2 * __fdividef(1.f, top * top));  // squares
-        const bool last = j == m - 1 || !(b2 > 1e-12f * sm.n2[0]) || prod < 1e-24f;
-        const float ib = last ? 0.f : rsqrtf(b2);
-        if (tid == 0) {
-            sm.al[j] = alpha;
-            sm.be[j] = last ? 0.f : b2 * ib;
-        }
-        if (last) {
-            k = j + 1;
-            break;
-        }
-        if (tid < kPad) sm.Q[j + 1][tid] = v * ib;
-        __syncthreads();
-    }
-    __syncthreads();
-
-    // ---- T's largest eigenvalue and its vector, by every thread alike
-    float f[kSteps], inv[kSteps], s[kSteps];
-    float theta, rest;
-    {
-        float al[kSteps], be[kSteps];
-        float lo = -INFINITY, hi = -INFINITY, sum = 0.f, bp = 0.f;
-#pragma unroll
-        for (int c = 0; c < kSteps; ++c) {
-            // past the space: a pivot of 1e30, which leaves its component zero
-            al[c] = c < k ? sm.al[c] : -1e30f;
-            be[c] = c < k ? sm.be[c] : 0.f;
-            sum += c < k ? al[c] : 0.f;
-            lo = fmaxf(lo, al[c]);
-            hi = fmaxf(hi, al[c] + bp + be[c]);
-            bp = be[c];
-        }
-        rest = trace - sum;
-        hi = hi * (1.f + 1e-6f);
-#pragma unroll 1
-        for (int round = 0; round < 4; ++round) {
-            const float x = lo + (hi - lo) * ((float)(lane + 1) * (1.f / 32.f));
-            float d = al[0] - x;
-            bool above = d < 0.f;
-#pragma unroll
-            for (int c = 1; c < kSteps; ++c) {
-                d = (al[c] - x) - __fdividef(be[c - 1] * be[c - 1], d);
-                above = above && d < 0.f;
+                        for (int c = 0; c <= j; ++c) v = fmaf(-sm.ca[c], sm.Q[c][tid], v);
+                        y[tid] = v;
+                    }
+                    __syncthreads();
+                }
             }
-            const unsigned mask = __ballot_sync(0xffffffffu, above) | 0x80000000u;
-            const int first = __ffs(mask) - 1;
-            const float nh = __shfl_sync(0xffffffffu, x, first);
-            const float nl = __shfl_sync(0xffffffffu, x, first > 0 ? first - 1 : 0);
-            lo = first > 0 ? nl : lo;
-            hi = nh;
+            float b2 = sm.n2[1], v = tid < kPad ? y[tid] : 0.f;
+#pragma unroll 4
+            for (int c = 0; c <= j; ++c) {
+                const float d = sm.cb[c];
+                b2 = fmaf(-d, d, b2);
+                if (tid < kPad) v = fmaf(-d, sm.Q[c][tid], v);
+            }
+            // The space is exhausted when what is left of the product is rounding,
+            // and large enough when the product of beta / theta (theta by the
+            // largest alpha so far) is: it bounds the leading Ritz vector's last
+            // component, its share of the residual, up to the gaps.
+            const float alpha = sm.ca[j] + sm.cb[j];
+            top = fmaxf(top, alpha);
+            prod *= fminf(1.f, b2 * __fdividef(1.f, top * top));  // squares
+            const bool last = j == m - 1 || !(b2 > 1e-12f * sm.n2[0]) || prod < 1e-24f;
+            const float ib = last ? 0.f : rsqrtf(b2);
+            if (tid == 0) {
+                sm.al[j] = alpha;
+                sm.be[j] = last ? 0.f : b2 * ib;
+            }
+            if (last) {
+                k = j + 1;
+                break;
+            }
+            if (tid < kPad) sm.Q[j + 1][tid] = v * ib;
+            __syncthreads();
         }
-        theta = hi;
-        tri_factor(al, be, theta, f, inv);
-#pragma unroll
-        for (int c = 0; c < kSteps; ++c) s[c] = 1.f;
-#pragma unroll 1
-        for (int it = 0; it < 2; ++it) {
-            tri_solve(f, inv, s);
-            float n2 = 0.f;
+        __syncthreads();
+
+        // ---- T's largest eigenvalue and its vector (a restart: the new part of
+        // it, (theta I - T') t = beta_0 ||v|| e_1 without the first row and column,
+        // which keeps its digits when beta_0 is small), by every thread alike
+        float f[kSteps], inv[kSteps], s[kSteps];
+        float theta, rest;
+        {
+            float al[kSteps], be[kSteps];
+            float lo = -INFINITY, hi = -INFINITY, sum = 0.f, bp = 0.f;
 #pragma unroll
             for (int c = 0; c < kSteps; ++c) {
-                s[c] *= 1e-4f;  // (the squares of 1e7 stay far inside FP32's range)
-                n2 = fmaf(s[c], s[c], n2);
+                // past the space: a pivot of 1e30, which leaves its component zero
+                al[c] = c < k ? sm.al[c] : -1e30f;
+                be[c] = c < k ? sm.be[c] : 0.f;
+                sum += c < k ? al[c] : 0.f;
+                lo = fmaxf(lo, al[c]);
+                hi = fmaxf(hi, al[c] + bp + be[c]);
+                bp = be[c];
             }
-            const float sc = rsqrtf(n2);
-#pragma unroll
-            for (int c = 0; c < kSteps; ++c) s[c] *= sc;
-        }
-        tri_factor(al, be, theta * (1.f + kShift), f, inv);
-    }
-    if (tid < kPad) {
-        float v = 0.f;
-#pragma unroll
-        for (int c = 0; c < kSteps; ++c)
-            if (c < k) v = fmaf(s[c], sm.Q[c][tid], v);
-        sm.vh[tid] = v;
-        sm.vl[tid] = 0.f;
-    }
-    __syncthreads();
-    const long long t1 = clock64();
-
-    // ---- refinement (double-float; v is not renormalised between steps)
-    const bool deflate = B > k;
-    const float theta_c = deflate ? rest / (float)(B - k) : 0.f;
-    dfl rho = {0.f, 0.f}, vv = {0.f, 0.f};
-    int it = 0;
-    bool converged = false;
+            rest = trace - sum;
+            hi = hi * (1.f + 1e-6f);
 #pragma unroll 1
-    for (;; ++it) {
-        // w = A v: the products split exactly by an FMA, summed by TwoSum,
-        // the small terms in FP32, at most 16 per chain
-        {
-            constexpr int kCh = kNJ / 16;
-            float sum[kCh], lo[kCh];
+            for (int round = 0; round < 4; ++round) {
+                const float x = lo + (hi - lo) * ((float)(lane + 1) * (1.f / 32.f));
+                float d = al[0] - x;
+                bool above = d < 0.f;
 #pragma unroll
-            for (int h = 0; h < kCh; ++h) sum[h] = lo[h] = 0.f;
-#pragma unroll
-            for (int u = 0; u < 16; ++u)
-#pragma unroll
-                for (int h = 0; h < kCh; ++h) {
-                    const int j = u + 16 * h;
-                    const float vh = sm.vh[j0 + j], vl = sm.vl[j0 + j];
-                    const float p = __fmul_rn(ch[j], vh);
-                    const float pe = __fmaf_rn(ch[j], vh, -p);
-                    float e;
-                    two_sum(sum[h], p, sum[h], e);
-                    lo[h] = __fadd_rn(lo[h], e);
-                    lo[h] = __fadd_rn(lo[h], pe);
-                    lo[h] = __fmaf_rn(ch[j], vl, lo[h]);
-                    lo[h] = __fmaf_rn(cl[j], vh, lo[h]);
+                for (int c = 1; c < kSteps; ++c) {
+                    d = (al[c] - x) - __fdividef(be[c - 1] * be[c - 1], d);
+                    above = above && d < 0.f;
                 }
-            if constexpr (kCh > 1) {
-                float e;
-                two_sum(sum[0], sum[1], sum[0], e);
-                lo[0] = __fadd_rn(__fadd_rn(lo[0], lo[1]), e);
+                const unsigned mask = __ballot_sync(0xffffffffu, above) | 0x80000000u;
+                const int first = __ffs(mask) - 1;
+                const float nh = __shfl_sync(0xffffffffu, x, first);
+                const float nl = __shfl_sync(0xffffffffu, x, first > 0 ? first - 1 : 0);
+                lo = first > 0 ? nl : lo;
+                hi = nh;
             }
-            sm.part[sl][rl] = make_float2(sum[0], lo[0]);
-        }
-        __syncthreads();
-        exchange(true);
-        const float2 *w = sm.x[par];
-        par ^= 1;
-        if (warp < kVW) {
-            const dfl v = {sm.vh[tid], sm.vl[tid]}, wi = {w[tid].x, w[tid].y};
-            const dfl tvv = df_xor_sum(df_mul(v, v), 32), tvw = df_xor_sum(df_mul(v, wi), 32);
-            if (lane == 0) sm.red4[warp] = make_float4(tvv.h, tvv.l, tvw.h, tvw.l);
-        }
-        __syncthreads();
-        {  // every warp forms the same rho from the same partials
-            const float4 q = sm.red4[lane % kVW];
-            vv = df_xor_sum({q.x, q.y}, kVW);
-            rho = df_div(df_xor_sum({q.z, q.w}, kVW), vv);
-        }
-        if (warp < kVW) {
-            const dfl pv = df_mul(rho, {sm.vh[tid], sm.vl[tid]});
-            const dfl r = df_add({w[tid].x, w[tid].y}, {-pv.h, -pv.l});
-            const float ri = __fadd_rn(r.h, r.l);
-            sm.r[tid] = ri;
-            const float r2 = warp_sum(ri * ri);
-            if (lane == 0) sm.red2[warp] = r2;
-        }
-        __syncthreads();
-        float rr = 0.f;
+            theta = hi;
+            const float a0 = al[0], b0 = be[0], xs = theta * (1.f + kMargin);
+            if (round) {
+                al[0] = -1e30f;
+                be[0] = 0.f;
+            }
+            tri_factor(al, be, xs, f, inv);
+            if (round) {
 #pragma unroll
-        for (int i = 0; i < kVW; ++i) rr += sm.red2[i];
-        const float tol = 1e-13f * fmaxf(fabsf(rho.h), dmax_s);
-        converged = rr <= tol * tol * vv.h;
-        if (converged || it == kMaxRefine) break;
-        if (warp < k) {
-            const float g = dot<kPad>(sm.Q[warp], sm.r, lane);
-            if (lane == 0) sm.ca[warp] = g;
+                for (int c = 0; c < kSteps; ++c) s[c] = 0.f;
+                s[1] = b0 * sqrtf(vv.h);
+                tri_solve(f, inv, s);
+                al[0] = a0;
+                be[0] = b0;
+            } else {
+#pragma unroll
+                for (int c = 0; c < kSteps; ++c) s[c] = 1.f;
+#pragma unroll 1
+                for (int i = 0; i < 2; ++i) {
+                    tri_solve(f, inv, s);
+                    float n2 = 0.f;
+#pragma unroll
+                    for (int c = 0; c < kSteps; ++c) {
+                        s[c] *= 1e-4f;  // (the squares of 1e7 stay far inside FP32's range)
+                        n2 = fmaf(s[c], s[c], n2);
+                    }
+                    const float sc = rsqrtf(n2);
+#pragma unroll
+                    for (int c = 0; c < kSteps; ++c) s[c] *= sc;
+                }
+            }
+            tri_factor(al, be, theta * (1.f + kShift), f, inv);
         }
-        __syncthreads();
         if (tid < kPad) {
-            const float den = rho.h - theta_c;
-            const float idc = deflate && fabsf(den) > 1e-3f * fabsf(rho.h) ? 1.f / den : 0.f;
-            float g[kSteps], y[kSteps];
-#pragma unroll
-            for (int c = 0; c < kSteps; ++c) y[c] = g[c] = c < k ? sm.ca[c] : 0.f;
-            tri_solve(f, inv, y);
-            float acc = sm.r[tid] * idc;
+            float v = 0.f;
 #pragma unroll
             for (int c = 0; c < kSteps; ++c)
-                if (c < k) acc = fmaf(fmaf(-g[c], idc, y[c]), sm.Q[c][tid], acc);
-            float sum, e;
-            two_sum(sm.vh[tid], acc, sum, e);
-            const dfl nv = fast_two_sum(sum, __fadd_rn(sm.vl[tid], e));
-            sm.vh[tid] = nv.h;
-            sm.vl[tid] = nv.l;
+                if (c < k) v = fmaf(s[c], sm.Q[c][tid], v);
+            if (round) {  // v += Q t
+                float sum, e;
+                two_sum(sm.vh[tid], v, sum, e);
+                const dfl nv = fast_two_sum(sum, __fadd_rn(sm.vl[tid], e));
+                sm.vh[tid] = nv.h;
+                sm.vl[tid] = nv.l;
+            } else {
+                sm.vh[tid] = v;
+                sm.vl[tid] = 0.f;
+            }
+        }
+        __syncthreads();
+        if (round == 0) t1 = clock64();
+
+        // ---- refinement (double-float; v is not renormalised between steps)
+        const bool deflate = B > k;
+        const float theta_c = deflate ? rest / (float)(B - k) : 0.f;
+        float e_now = 0.f, rn = 0.f;
+#pragma unroll 1
+        for (;; ++it) {
+            // w = A v: the products split exactly by an FMA, summed by TwoSum,
+            // the small terms in FP32, at most 16 per chain
+            {
+                constexpr int kCh = kNJ / 16;
+                float sum[kCh], lo[kCh];
+#pragma unroll
+                for (int h = 0; h < kCh; ++h) sum[h] = lo[h] = 0.f;
+#pragma unroll
+                for (int u = 0; u < 16; ++u)
+#pragma unroll
+                    for (int h = 0; h < kCh; ++h) {
+                        const int j = u + 16 * h;
+                        const float vh = sm.vh[j0 + j], vl = sm.vl[j0 + j];
+                        const float p = __fmul_rn(ch[j], vh);
+                        const float pe = __fmaf_rn(ch[j], vh, -p);
+                        float e;
+                        two_sum(sum[h], p, sum[h], e);
+                        lo[h] = __fadd_rn(lo[h], e);
+                        lo[h] = __fadd_rn(lo[h], pe);
+                        lo[h] = __fmaf_rn(ch[j], vl, lo[h]);
+                        lo[h] = __fmaf_rn(cl[j], vh, lo[h]);
+                    }
+                if constexpr (kCh > 1) {
+                    float e;
+                    two_sum(sum[0], sum[1], sum[0], e);
+                    lo[0] = __fadd_rn(__fadd_rn(lo[0], lo[1]), e);
+                }
+                sm.part[sl][rl] = make_float2(sum[0], lo[0]);
+            }
+            __syncthreads();
+            exchange(true);
+            const float2 *w = sm.x[par];
+            par ^= 1;
+            if (warp < kVW) {
+                const dfl v = {sm.vh[tid], sm.vl[tid]}, wi = {w[tid].x, w[tid].y};
+                const dfl tvv = df_xor_sum(df_mul(v, v), 32), tvw = df_xor_sum(df_mul(v, wi), 32);
+                if (lane == 0) sm.red4[warp] = make_float4(tvv.h, tvv.l, tvw.h, tvw.l);
+            }
+            __syncthreads();
+            {  // every warp forms the same rho from the same partials
+                const float4 q = sm.red4[lane % kVW];
+                vv = df_xor_sum({q.x, q.y}, kVW);
+                rho = df_div(df_xor_sum({q.z, q.w}, kVW), vv);
+            }
+            if (warp < kVW) {
+                const dfl pv = df_mul(rho, {sm.vh[tid], sm.vl[tid]});
+                const dfl r = df_add({w[tid].x, w[tid].y}, {-pv.h, -pv.l});
+                const float ri = __fadd_rn(r.h, r.l);
+                sm.r[tid] = ri;
+                const float r2 = warp_sum(ri * ri);
+                if (lane == 0) sm.red2[warp] = r2;
+            }
+            __syncthreads();
+            float rr = 0.f;
+#pragma unroll
+            for (int i = 0; i < kVW; ++i) rr += sm.red2[i];
+            const float tol = 1e-13f * fmaxf(fabsf(rho.h), dmax_s);
+            converged = rr <= tol * tol * vv.h;
+            rn = sqrtf(rr);
+            e_now = rr / vv.h;
+            // one restart after another once the first space has given what it
+            // has (NaN counts as slow)
+            if (converged || round || !(e_now * kSlow < e_last)) break;
+            e_last = e_now;
+            if (warp < k) {
+                const float g = dot<kPad>(sm.Q[warp], sm.r, lane);
+                if (lane == 0) sm.ca[warp] = g;
+            }
+            __syncthreads();
+            if (tid < kPad) {
+                const float den = rho.h - theta_c;
+                const float idc = deflate && fabsf(den) > 1e-3f * fabsf(rho.h) ? 1.f / den : 0.f;
+                float g[kSteps], y[kSteps];
+#pragma unroll
+                for (int c = 0; c < kSteps; ++c) y[c] = g[c] = c < k ? sm.ca[c] : 0.f;
+                tri_solve(f, inv, y);
+                float acc = sm.r[tid] * idc;
+#pragma unroll
+                for (int c = 0; c < kSteps; ++c)
+                    if (c < k) acc = fmaf(fmaf(-g[c], idc, y[c]), sm.Q[c][tid], acc);
+                float sum, e;
+                two_sum(sm.vh[tid], acc, sum, e);
+                const dfl nv = fast_two_sum(sum, __fadd_rn(sm.vl[tid], e));
+                sm.vh[tid] = nv.h;
+                sm.vl[tid] = nv.l;
+            }
+            __syncthreads();
+        }
+        if (converged) break;
+        if (round && !(e_now * kSlow < e_round)) ++stalled;
+        if (stalled == 2 || round == kMaxRounds || B < 2) break;
+        e_round = e_now;
+        ++it;
+        // ---- restart: the columns v / ||v|| and r / ||r|| (from the double-float
+        // residual: FP32's product would not know it), T's first row
+        if (tid < kPad) sm.Q[0][tid] = sm.vh[tid] * rsqrtf(vv.h);
+        __syncthreads();
+        {
+            const float g = dot<kPad>(sm.Q[0], sm.r, lane);
+            if (tid < kPad) sm.Q[1][tid] = fmaf(-g, sm.Q[0][tid], sm.r[tid]);
+        }
+        __syncthreads();
+        {
+            const float n2 = dot<kPad>(sm.Q[1], sm.Q[1], lane);
+            __syncthreads();
+            if (tid < kPad) sm.Q[1][tid] *= rsqrtf(n2);
+            if (tid == 0) {
+                sm.al[0] = rho.h;
+                sm.be[0] = rn * rsqrtf(vv.h);
+            }
         }
         __syncthreads();
     }
