@@ -172,9 +172,10 @@ hsc_status hsc_pca_one_band(hsc_ctx *ctx, const float *cube, int B, int H, int W
  * n_pc leading eigenvectors of the covariance, each refined to the residual
  * bound of hsc_pca_one_band and signed by the same rule (v_1 is
  * hsc_pca_one_band's), and out_j = v_j^T (x - mu). The eigenvectors beyond
- * the first are refined from the 16 basis columns of the first sweep, so a
- * component whose eigenvalue is not separated from its neighbours may not
- * converge (HSC_ERR_NOT_CONVERGED at hsc_sync).
+ * the first are refined from the eigensolver's 16 basis columns (from the
+ * columns of its full sweeps where the lead needed them), so a component whose
+ * eigenvalue is not separated from its neighbours may not converge
+ * (HSC_ERR_NOT_CONVERGED at hsc_sync).
  *   n_pc     1 .. min(HSC_MAX_PC, B)
  *   flags    0 or HSC_CUBE_BIP
  *   out      n_pc x H x W float32 (device, required); out_0 equals the raw

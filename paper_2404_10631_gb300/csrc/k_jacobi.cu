@@ -1370,30 +1370,43 @@ if (presweep) {
     // ---- further eigenvectors (multi-PC projection): v_j for j = 1 .. n_vec-1,
     // each refined from basis column j (the j-th Ritz vector, or the j-th
     // largest diagonal's column after the sweep) by the same deflated
-    // correction aimed at column j, then the same sign rule. Phase 0's basis
-    // only (the fallback rebuilds none).
-    if (prm.n_vec > 1 && !fell_back) {
-        const bool sm_basis = prm.use_smem && !kPacked;
+    // correction aimed at column j, then the same sign rule. After the
+    // fallback: from the column of the next largest eigenvalue, as its lead.
+    if (prm.n_vec > 1) {
+        const bool sm_basis = prm.use_smem && !kPacked && !fell_back;
         const size_t xo = jac_phase0_floats(n);
-        const float *bas = sm_basis ? smem + xo : X;
-        const float2 *c2p = sm_basis ? reinterpret_cast<const float2 *>(smem)
-                                     : (prm.use_smem ? Cs2 : C2);
+        const float *bas = fell_back ? Vt : sm_basis ? smem + xo : X;
+        const float2 *c2p = fell_back  ? C2
+                            : sm_basis ? reinterpret_cast<const float2 *>(smem)
+                                       : (prm.use_smem ? Cs2 : C2);
         float2 *partp = sm_basis ? reinterpret_cast<float2 *>(smem + xo + (size_t)kBasis * ld) : part;
-        for (int j = 1; j < prm.n_vec && j < m; ++j) {
+        const int ncol = fell_back ? B : m;
+        for (int j = 1; j < prm.n_vec && j < ncol; ++j) {
+            if (fell_back && tid == 0) {  // after s_lead in (eigenvalue, smaller column) order
+                const int was = s_lead;
+                int next = -1;
+                for (int q = 0; q < B; ++q) {
+                    const bool after = th[q] < th[was] || (th[q] == th[was] && q > was);
+                    if (after && (next < 0 || th[q] > th[next])) next = q;
+                }
+                s_lead = next < 0 ? was : next;  // (NaN eigenvalues: any)
+            }
             __syncthreads();
+            const int col = fell_back ? s_lead : j;
             for (int ii = tid; ii < B; ii += nthr) {
-                vh[ii] = bas[(size_t)j * ld + ii];
+                vh[ii] = bas[(size_t)col * ld + ii];
                 vl[ii] = 0.f;
             }
             __syncthreads();
-            const int it = refine(bas, m, j, deflate, theta_c, c2p, partp);
+            const int it = refine(bas, ncol, col, !fell_back && deflate, fell_back ? 0.f : theta_c, c2p,
+                                  partp);
             if (it > kMaxRefine) {
                 // not converged (an eigenvalue inside a cluster): report it and
                 // return the basis column itself, finite, with its estimate
                 if (tid == 0) atomicOr(&ctl->status, ST_NOT_CONVERGED);
                 __syncthreads();
                 for (int ii = tid; ii < B; ii += nthr) {
-                    vh[ii] = bas[(size_t)j * ld + ii];
+                    vh[ii] = bas[(size_t)col * ld + ii];
                     vl[ii] = 0.f;
                 }
                 float sq = 0.f;
@@ -1401,7 +1414,7 @@ if (presweep) {
                 sq = block_sumf(sq, fred);
                 if (tid == 0) {
                     s_vv = dfl{sq, 0.f};
-                    s_rho = dfl{th[j], 0.f};
+                    s_rho = dfl{th[col], 0.f};
                 }
             }
             finish(prm.vk + (size_t)j * B, prm.vkf + (size_t)j * B, prm.lamk + j);
