@@ -367,7 +367,7 @@ hsc_status hsc_pca_diagnostics(hsc_ctx *ctx, int32_t *sweeps, int32_t *refine_it
 /* Autotuner (launch parameters that change speed, never results): times the
  * candidates of the tensor-core Gram's TMA staging depth (3 or 4 stages;
  * B <= 128), of the projection/SVM pass's launch shape (1 or 4 pixels per
- * thread, the latter meaning 2 with 2, 3 or 5 classes, x 2, 4, 8 or 16 CTAs
+ * thread, the latter meaning 2 with 2 or 3 classes, x 2, 4, 8 or 16 CTAs
  * per SM) and, given KNN parameters with
  * lambda > 0 and the pruned search, of the pruned walk's warps per CTA
  * (variants 0: 4, 1: 1, 2: 2, 3: 8, 4: 4, 5: 6; every pixel's neighbour

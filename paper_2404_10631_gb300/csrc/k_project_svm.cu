@@ -37,9 +37,10 @@ constexpr int kFrameThreads = 128;
 // kF64: the coupling to FP64-level accuracy (a kernel of its own: the refined
 // solve is several times the code of the plain one). From five classes on it
 // is held to 128 registers, four CTAs of 128 threads per SM: 415 x 513 x 128, 7
-// classes 95 -> 71 us, 8 classes 119 -> 97 us.
+// classes 95 -> 71 us, 8 classes 119 -> 97 us; so are four pixels of five
+// classes (1000 x 1000 x 100 109 -> 96 us).
 template <int KC, int PX, bool kVec, bool kF64>
-__global__ void __launch_bounds__(kThreads, kF64 && KC >= 5 && PX == 1 ? 2 : 0)
+__global__ void __launch_bounds__(kThreads, (kF64 && KC >= 5 && PX == 1) || (KC == 5 && PX == 4) ? 2 : 0)
 project_svm_kernel(const float *__restrict__ cube, int B, long N,
                    const float *__restrict__ v1f, const float *__restrict__ muf,
                    const float *__restrict__ w, const float *__restrict__ bias,
@@ -177,15 +178,24 @@ cudaError_t launch_project_svm(const float *cube, int B, long N, const float *v1
 {
     const int k = (probs != nullptr && model != nullptr) ? model->n_classes : 0;
     const bool vec = (N % 4 == 0) && ((reinterpret_cast<uintptr_t>(cube) & 15u) == 0);
-    // Pixels per thread. Few classes: 4 (16-byte loads) or, with 2, 3 or 5, 2;
+    // Pixels per thread. Few classes: 4 (16-byte loads) or, with 2 or 3, 2;
     // many: one (15 accumulators per pixel with 6 classes: 4 pixels leave too
-    // few warps). Under 64 K pixels one as well: the threads are what is short.
-    // Measured, 4 / 2 / 1 pixels: 416 x 512 x 128, 4 classes 27.2 / 29.0 / 32.8
-    // us; 1000 x 1000 x 100, 3 classes 72 / 66 / 77; 509 x 401 x 100, 6 classes
-    // 57 / 49 / 43; 416 x 512 x 128, 8 classes 132 / 92 / 76; 200 x 200 x 128, 4
-    // classes 17.2 / 13.2 / 13.1; 48 x 48 x 125, 4 classes 16.0 / 12.1 / 10.4.
-    if (px == 0) px = N < 65536 || k >= 6 ? 1 : 4;
-    if (px == 4 && (k == 2 || k == 3 || k == 5)) px = 2;
+    // few warps). Under 64 K pixels one as well (the threads are what is short),
+    // under 96 K one with 4 classes and two with 5.
+    // Measured, 4 / 2 / 1 pixels: 2 classes 256 x 257 x 128 8.8 / 6.6 / 7.3 us,
+    // 416 x 512 x 128 17.0 / 15.2 / 19.5; 3 classes 1000 x 1000 x 100 66 / 73 /
+    // 97, 415 x 513 x 128 22.1 / 18.3 / 22.4; 4 classes 256 x 257 x 128 12.8 /
+    // 9.5 / 10.4, 300 x 300 x 224 27.5 / 18.7 / 18.1, 340 x 352 x 128 16.3 / 19.3
+    // / 19.1, 416 x 512 x 128 22.4 / 25.5 / 25.8; 5 classes 256 x 257 x 128 15.7
+    // / 11.4 / 12.4, 300 x 300 x 224 34.7 / 23.4 / 23.2, 340 x 352 x 128 21.1 /
+    // 24.3 / 24.2, 1000 x 1000 x 100 96 / 116 / 134; 6 classes 509 x 401 x 100 57
+    // / 49 / 43; 8 classes 416 x 512 x 128 132 / 92 / 76.
+    if (px == 0) {
+        if (N < 65536 || k >= 6) px = 1;
+        else if (N < 98304 && (k == 4 || k == 5)) px = k == 4 && !couple_f64 ? 1 : 2;
+        else px = 4;
+    }
+    if (px == 4 && (k == 2 || k == 3)) px = 2;
     // the refined coupling solves, by their code and registers: two pixels at
     // most, one from five classes on (415 x 513 x 128, two / one: 4 classes 31 /
     // 38 us, 5 classes 50 / 42, 6 classes 64 / 57, 8 classes 141 / 97)
