@@ -8,7 +8,9 @@
 // order, a lane per pixel: e does not decrease on either side (a rounded
 // difference and its rounded square are monotone), so the next nearest is
 // always one of two. Entries of equal e (equal values, values on both sides,
-// or values whose rounded distances agree) are one group, listed by index.
+// or values whose rounded distances agree) are one group, listed by index; a
+// group of many values (distances that underflow or overflow to one e) is
+// taken from the window in index order, which stops at the K-th.
 // O(n log^2 n) per row and O(K) per pixel, where the full scan
 // (knn_kernel) forms n keys per pixel and, without a spatial term to bound
 // them, keeps replacing its candidates. Measured: 208 x 256, K = 16, 7 rows
@@ -28,6 +30,11 @@ namespace hsc {
 namespace {
 
 constexpr int kThreads = 512;
+// Runs of a group that give the full list nothing before the group is taken in
+// index order instead. Two runs, one on either side, are a group of ordinary
+// values; hundreds are one where the squared distances underflow or overflow
+// (1 x 4096, values of 1e-24, K = 16: 39 ms run by run, 0.53 ms this way).
+constexpr int kPastRuns = 16;
 
 // Entries are (ordered value key << 32 | index).
 __device__ __forceinline__ float value_of(unsigned long long x)
@@ -107,6 +114,7 @@ knn_value_kernel(const float *__restrict__ I, const float *__restrict__ P, int H
             const float e = (lf >= 0 && !(el > er)) || rt >= n ? el : er;
             m0 = m;
             bool moved = false;
+            int past = 0;  // runs all of whose indices are out
             // runs of one value, the indices of each ascending
             while (lf >= 0 && dist(lf) == e) {
                 const unsigned v = (unsigned)(s[lf] >> 32);
@@ -116,6 +124,7 @@ knn_value_kernel(const float *__restrict__ I, const float *__restrict__ P, int H
                 while (i <= lf && put((int)(unsigned)s[i])) ++i;
                 lf = first - 1;
                 moved = true;
+                if (i == first && ++past > kPastRuns) break;
             }
             while (rt < n && dist(rt) == e) {
                 const unsigned v = (unsigned)(s[rt] >> 32);
@@ -123,6 +132,16 @@ knn_value_kernel(const float *__restrict__ I, const float *__restrict__ P, int H
                 while (rt < n && (unsigned)(s[rt] >> 32) == v && (in = put((int)(unsigned)s[rt]))) ++rt;
                 if (!in) rt = v == 0xffffffffu ? n : lower_bound(s, n, v + 1u);
                 moved = true;
+                if (!in && ++past > kPastRuns) break;
+            }
+            if (past > kPastRuns) {  // the group fills the list: its first by a scan in index order
+                m = m0;
+                for (int q = q0; m < K && q < q0 + n; ++q) {
+                    const float v = __ldg(I + q);
+                    const float d = __fsub_rn(Ip, v == 0.f ? 0.f : v);
+                    if (__fmul_rn(d, d) == e) sel[m++] = q;
+                }
+                break;
             }
             if (!moved) {  // NaN: no e equals itself; any entry will do
                 put((int)(unsigned)s[lf >= 0 ? lf : rt]);
