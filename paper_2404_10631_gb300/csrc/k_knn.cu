@@ -994,9 +994,11 @@ knn_redo_kernel(const float *__restrict__ I, const float *__restrict__ P, int H,
 {
     extern __shared__ float sm[];
     pdl_wait();
-    pdl_next();
     const long N = (long)H * W;
-    if (*(volatile unsigned *)&ctl->knn_redo == 0u) return;
+    if (*(volatile unsigned *)&ctl->knn_redo == 0u) {
+        pdl_next();  // (with work to do it may take milliseconds)
+        return;
+    }
     for (long base = (long)blockIdx.x * kRedoThreads; base < N;
          base += (long)gridDim.x * kRedoThreads) {
         const long p = base + threadIdx.x;
