@@ -955,19 +955,22 @@ __device__ __noinline__ void redo_pixel(const float *__restrict__ I, const float
 }
 
 
-constexpr int kRedoCap = 32;           // undecided keys per lane in box_pixel
-// box_pixel for the second pass, a warp together (todo: this lane has a
-// pixel): true where the pixel is left.
+
+// box_pixel for the second pass, a warp together (todo: this lane has a pixel,
+// far: only the unbounded walk can finish it): true where the pixel is left.
 template <int KC>
-__device__ __forceinline__ bool redo_box(const TileFrame &f, bool todo, long p, int K, int R,
-                                         float lam, float *sm)
+__device__ __forceinline__ bool redo_box(const TileFrame &f, bool todo, bool far, long p, int K,
+                                         int R, float lam, float *sm)
 {
+    far = far && todo;
     const Buf buf = {(uint32_t)__cvta_generic_to_shared(sm) + 4u * (threadIdx.x & 31)};
     const float l2 = lam * lam;
-    const int q = todo ? (int)p : -1;
-    unsigned ev = f.P4 ? box_pixel<KC, true>(f, q, K, R, l2, buf, kRedoCap)
-                       : box_pixel<KC, false>(f, q, K, R, l2, buf, kRedoCap);
-    const bool left = ev == ~0u;
+    const int q = todo && !far ? (int)p : -1;
+    unsigned ev = 0u;
+    if (__any_sync(0xffffffffu, q >= 0))
+        ev = f.P4 ? box_pixel<KC, true>(f, q, K, R, l2, buf, kRedoCap)
+                  : box_pixel<KC, false>(f, q, K, R, l2, buf, kRedoCap);
+    const bool left = far || ev >= kLeftKeys;
     const unsigned n = __popc(__ballot_sync(0xffffffffu, left));
     ev = __reduce_add_sync(0xffffffffu, left ? 0u : ev);
     if ((threadIdx.x & 31) == 0) {
@@ -979,7 +982,9 @@ __device__ __forceinline__ bool redo_box(const TileFrame &f, bool todo, long p, 
 
 // Completes the pixels the pruned walk left with the sentinel label, 32
 // consecutive pixels per warp (left pixels come in clusters along the borders
-// of regions): box_pixel, and for what that leaves a walk from global memory
+// of regions): box_pixel where its larger buffer holds the undecided keys (not
+// tried for others: 416 x 512 of noise, K = 40, lambda 0.1 4.29 -> 4.06 ms, 0.25
+// 1.43 -> 1.39 ms), and for what that leaves a walk from global memory
 // (the table in increasing s, then row by row over the
 // rest of the window, or of the disk s_term <= tau once K are in), keeping
 // every key <= tau in a buffer of K + 32 (compacted to the best K when full),
@@ -1002,10 +1007,12 @@ knn_redo_kernel(const float *__restrict__ I, const float *__restrict__ P, int H,
     for (long base = (long)blockIdx.x * kRedoThreads; base < N;
          base += (long)gridDim.x * kRedoThreads) {
         const long p = base + threadIdx.x;
-        bool todo = p < N && labels[p] == kRedoLabel;
+        const int label = p < N ? labels[p] : 0;
+        const bool far = label == kRedoFarLabel;
+        bool todo = far || label == kRedoLabel;
         if (!__any_sync(0xffffffffu, todo)) continue;
         if (!nbr) {
-            todo = redo_box<KC>({I, P, P4, O, labels, ctl, N, H, W}, todo, p, K, R, lam, sm);
+            todo = redo_box<KC>({I, P, P4, O, labels, ctl, N, H, W}, todo, far, p, K, R, lam, sm);
             __syncwarp();  // sm is shared with redo_pixel's buffers
         }
         if (todo) redo_pixel<KC>(I, P, H, W, K, R, lam, O, labels, nbr, ctl, p, sm, P4);
@@ -1039,9 +1046,9 @@ knn_redo_batch_kernel(const BatchFrame *__restrict__ frames, int K, int R, float
         const unsigned i = i0 + threadIdx.x;
         bool todo = i < n;
         const int2 fp = redo_list[todo ? i : 0];
-        const BatchFrame &fr = frames[fp.x];
+        const BatchFrame &fr = frames[fp.x < 0 ? ~fp.x : fp.x];
         todo = redo_box<KC>({fr.I, fr.P, fr.P4, fr.O, fr.labels, fr.ctl, fr.N, fr.H, fr.W}, todo,
-                            (long)fp.y, K, R, lam, sm);  // (a frame per lane)
+                            fp.x < 0, (long)fp.y, K, R, lam, sm);  // (a frame per lane)
         __syncwarp();
         if (todo)
             redo_pixel<KC>(fr.I, fr.P, fr.H, fr.W, K, R, lam, fr.O, fr.labels, nullptr, fr.ctl,

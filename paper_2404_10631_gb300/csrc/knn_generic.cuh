@@ -154,8 +154,10 @@ __device__ __forceinline__ int isqrt_d(int x)
 // s < s_K whose key is below L as they come (canonical order) and lists the
 // others. tau = L + e_max over the candidates seen bounds the K-th key; where
 // it reaches past s_K the ring up to it is walked the same way. The K - m
-// smallest of the list complete the set. Returns the keys kept, or ~0u: not
-// finished (more than cap undecided keys, or a disk beyond the table's).
+// smallest of the list complete the set. Returns the keys kept, or that the
+// pixel is not finished: kLeftKeys (more than cap undecided keys, kRedoCap
+// hold them) or kLeftFar (more still, or a disk beyond the table's).
+constexpr unsigned kLeftFar = ~0u, kLeftKeys = ~0u - 1u;
 template <int KC, bool kP4>
 __device__ __forceinline__ unsigned box_pixel(const TileFrame &f, int p, int K, int R, float l2,
                                               Buf buf, int cap)
@@ -281,7 +283,10 @@ __device__ __forceinline__ unsigned box_pixel(const TileFrame &f, int p, int K, 
     const int s1w = __reduce_max_sync(kAll, s1);
     if (s1w >= 0) walk(std::true_type(), sK, s1, s1w);
     const int need = K - m;
-    if (!ok || n > cap || n < need) return on ? ~0u : 0u;  // (n < need: NaN in the map)
+    if (!ok || n > cap || n < need) {  // (n < need: NaN in the map)
+        if (!on) return 0u;
+        return ok && n > cap && n <= kRedoCap ? kLeftKeys : kLeftFar;
+    }
 #pragma unroll 1
     for (int a = 0; a < need; ++a) {  // the smallest of entries a .. n-1 to place a
         const Key first = buf.get(a);

@@ -17,8 +17,12 @@ constexpr int kTabDr = 16;             // |dr| <= 16: windows of up to 32 rows
 constexpr int kTabDc = 20;             // |dc| <= 20 follows from kTabR2
 constexpr int kTabCap = 1200;
 
-// Label of a pixel left to the redo pass.
+// Labels of a pixel left to the redo pass: box_pixel with its larger buffer may
+// finish it, or (kRedoFarLabel) only the unbounded walk can. The batch's list
+// holds the latter's frame as ~frame.
 constexpr int kRedoLabel = -2147483647 - 1;
+constexpr int kRedoFarLabel = kRedoLabel + 1;
+constexpr int kRedoCap = 32;  // undecided keys per lane in the redo pass's box_pixel
 
 struct Key {
     float hi, lo;

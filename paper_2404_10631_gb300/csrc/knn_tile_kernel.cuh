@@ -21,7 +21,7 @@
 // own warp, a row at a time (left to a second kernel they came to it in
 // clusters, a few warps with several rows each: 509 x 401, K = 24, lambda 0.5
 // 60 us). Pixels with too many undecided keys there are left to the second
-// pass (label kRedoLabel).
+// pass (labels kRedoLabel, kRedoFarLabel).
 //
 // Measured, walk and second pass together, against one pixel per lane with
 // every candidate of the disk keyed and P gathered by dependent loads:
@@ -307,12 +307,12 @@ knn_tile_kernel(const __grid_constant__ TileArgs a)
     const int K = a.K, W = f.W;
     const TileGeom g = tile_geom(f.H, f.W, a.rad, a.cut, nw);
     unsigned evals = 0, redo = 0;
-    auto leave = [&](int p) {  // to the second pass
+    auto leave = [&](int p, bool far) {  // to the second pass
         ++redo;
-        f.labels[p] = kRedoLabel;
+        f.labels[p] = far ? kRedoFarLabel : kRedoLabel;
         if (a.frames) {
             const unsigned i = atomicAdd(&a.frames[0].ctl->knn_redo_list, 1u);
-            if (i < a.redo_cap) a.redo_list[i] = make_int2(frame, p);
+            if (i < a.redo_cap) a.redo_list[i] = make_int2(far ? ~frame : frame, p);
         }
     };
     // the pixels that box_pixel takes: this lane's border pixel, or the rows
@@ -346,8 +346,8 @@ knn_tile_kernel(const __grid_constant__ TileArgs a)
     for (int v = 0; v < passes; ++v) {
         const int p = p0 >= 0 ? p0 + v * W : -1;
         const unsigned ev = box_pixel<KC, kP4>(f, p, K, a.R, l2, buf, kTileCap);
-        if (ev != ~0u) evals += ev;
-        else leave(p);
+        if (ev < kLeftKeys) evals += ev;
+        else leave(p, ev == kLeftFar);
     }
     // the counters: keys formed, pixels left to the second pass
 #pragma unroll
