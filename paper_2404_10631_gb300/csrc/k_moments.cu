@@ -17,7 +17,8 @@
 namespace hsc {
 namespace {
 
-constexpr int kGramThreads = 288;
+constexpr int kGramThreads = 288;     // FP32-pipe Gram, one CTA per SM
+constexpr int kGramFewThreads = 256;  // the same, two CTAs per SM
 constexpr int kGramChunk = 32;   // pixels staged per step
 constexpr int kTile = 8;         // 8x8 accumulator tile per thread
 
@@ -235,16 +236,18 @@ __device__ __forceinline__ dfl cov_entry(float g, float gl, dfl inv, dfl db, dfl
 // in two planes (b % 8 < 4 and >= 4), so that the lanes of a warp, which share
 // ti and have consecutive tj, read consecutive 16-byte units; Bp / 4 + 1 is
 // odd, so the lanes of a staging store (one pixel each) fall into different
-// banks too. kAhead (up to 256 bands): the next chunk's values are loaded into
-// registers before this one's sums; above, loaded and stored in turn.
-// Measured (means and covariance): 1023 x 1024 x 256 10.3 -> 4.8 ms, 333 x 500 x
-// 224 1.51 -> 0.76 ms, 60 x 60 x 256 301 -> 230 us, 40 x 41 x 129 205 -> 141 us,
-// against 256 tiles per CTA of the whole square, loaded and stored in turn
-// with 4-way bank conflicts. The FMAs are a third of the issue slots: what is
-// left is the wait for the loads (nine warps per SM) and, with few
-// partitions, the last round of CTAs.
-template <bool kAhead>
-__global__ void __launch_bounds__(kGramThreads, 1)
+// banks too. Two forms: one CTA of 288 threads per SM, the next chunk's values
+// loaded into registers before this one's sums (kAhead; above 256 bands they
+// are too many: loaded and stored in turn), and two CTAs of 256 threads, which
+// wait for one another's loads (launch_moments says which).
+// Measured (means and covariance), the first form against 256 tiles per CTA of
+// the whole square, loaded and stored in turn with 4-way bank conflicts: 1023 x
+// 1024 x 256 10.3 -> 4.8 ms, 333 x 500 x 224 1.51 -> 0.76 ms, 60 x 60 x 256 301
+// -> 230 us, 40 x 41 x 129 205 -> 141 us. The FMAs are a third of the issue
+// slots: what is left is the wait for the loads (nine warps per SM) and, with
+// few partitions, the last round of CTAs.
+template <bool kAhead, int kThr, int kMin>
+__global__ void __launch_bounds__(kThr, kMin)
 gram_partial_kernel(const float *__restrict__ cube, int B, int Bp, long N, int per_cta,
                     const float *__restrict__ shift, float *__restrict__ gram_part,
                     float *__restrict__ sum_part, Control *ctl)
@@ -267,7 +270,7 @@ gram_partial_kernel(const float *__restrict__ cube, int B, int Bp, long N, int p
     const int tj = has_tile ? tile - ti * (ti + 1) / 2 : 0;
     const bool do_sums = (blockIdx.y == 0);
 
-    for (int b = tid; b < Bp; b += kGramThreads) sh[b] = (b < B) ? shift[b] : 0.f;
+    for (int b = tid; b < Bp; b += kThr) sh[b] = (b < B) ? shift[b] : 0.f;
 
     long per = (N + gridDim.x - 1) / gridDim.x;
     long p0 = (long)blockIdx.x * per, p1 = p0 + per;
@@ -278,8 +281,8 @@ gram_partial_kernel(const float *__restrict__ cube, int B, int Bp, long N, int p
     for (int a = 0; a < kTile; ++a)
 #pragma unroll
         for (int c = 0; c < kTile; ++c) acc[a][c] = 0.f;
-    // running sums of the bands tid + kGramThreads q
-    constexpr int kSums = kAhead ? 1 : (1024 + kGramThreads - 1) / kGramThreads;
+    // running sums of the bands tid + kThr q
+    constexpr int kSums = kAhead ? 1 : (1024 + kThr - 1) / kThr;
     float bsum[kSums];
 #pragma unroll
     for (int q = 0; q < kSums; ++q) bsum[q] = 0.f;
@@ -287,8 +290,8 @@ gram_partial_kernel(const float *__restrict__ cube, int B, int Bp, long N, int p
     const float *ra = Yt + ti * 4, *rb = Yt + tj * 4;
 
     // staging: a lane per pixel, four bands of it per store; quad j of a warp
-    constexpr int kWarps = kGramThreads / 32;
-    constexpr int kQuads = (256 / 4 + kWarps - 1) / kWarps;
+    constexpr int kWarps = kThr / 32;
+    constexpr int kQuads = kAhead ? (256 / 4 + kWarps - 1) / kWarps : 1;
     const int warp = tid >> 5, lane = tid & 31;
     auto load = [&](float (&x)[4], int q, long p) {
 #pragma unroll
@@ -331,7 +334,7 @@ gram_partial_kernel(const float *__restrict__ cube, int B, int Bp, long N, int p
         if (do_sums) {
 #pragma unroll
             for (int q = 0; q < kSums; ++q) {
-                const int b = tid + kGramThreads * q;
+                const int b = tid + kThr * q;
                 if (b < Bp) {
                     const float *col = Yt + ((b >> 2) & 1) * half + (b >> 3) * 4 + (b & 3);
                     float t = 0.f;
@@ -375,7 +378,7 @@ gram_partial_kernel(const float *__restrict__ cube, int B, int Bp, long N, int p
     if (do_sums) {
 #pragma unroll
         for (int q = 0; q < kSums; ++q) {
-            const int b = tid + kGramThreads * q;
+            const int b = tid + kThr * q;
             if (b < B) sum_part[(size_t)blockIdx.x * B + b] = bsum[q];
         }
     }
@@ -561,7 +564,7 @@ static cudaError_t launch_reductions(int B, long N, int n_part, const PcaScratch
 {
     const double inv_N = 1.0 / (double)N;
     const long BB = (long)B * B;
-return launch_pdl(gram_reduce_kernel, dim3((unsigned)((BB + kRedEntries - 1) / kRedEntries)),
+    return launch_pdl(gram_reduce_kernel, dim3((unsigned)((BB + kRedEntries - 1) / kRedEntries)),
                       dim3(kRedEntries * kRedSlices), 0, st, B, inv_N, n_part, s.gram_part,
                       s.sum_part, s.shift, s.mu, s.C, s.C2);
 }
@@ -591,15 +594,24 @@ cudaError_t launch_moments(const float *cube, int B, long N, const PcaScratch &s
     const int Bp = (B + kTile - 1) / kTile * kTile;
     const int nt = Bp / kTile;
     const int tiles = nt * (nt + 1) / 2;
-    const int groups = (tiles + kGramThreads - 1) / kGramThreads;
+    // Up to 176 bands (one group of tiles) two CTAs per SM, above 112 only where
+    // there are partitions for them. Measured, first form / second: 1001 x 999 x
+    // 16 556 / 234 us (the whole square's kernel: 255), 501 x 401 x 48 209 / 94
+    // (162), 201 x 203 x 8 95 / 79 (84), x 100 131 / 114, x 128 169 / 201, 701 x
+    // 701 x 128 620 / 381, 333 x 501 x 176 461 / 333.
+    const bool two = Bp <= 112 || (Bp <= 176 && s.n_part > sm_count);
+    const int thr = two ? kGramFewThreads : kGramThreads;
+    const int groups = (tiles + thr - 1) / thr;
     const int per_cta = (tiles + groups - 1) / groups;
     size_t smem = sizeof(float) * ((size_t)kGramChunk * (Bp + 4) + Bp);
-    auto kern = Bp <= 256 ? gram_partial_kernel<true> : gram_partial_kernel<false>;
+    auto kern = two         ? gram_partial_kernel<false, kGramFewThreads, 2>
+                : Bp <= 256 ? gram_partial_kernel<true, kGramThreads, 1>
+                            : gram_partial_kernel<false, kGramThreads, 1>;
     if (smem > 48 * 1024)
         cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     dim3 grid(s.n_part, groups);
     const cudaError_t ge =
-        launch_pdl(kern, grid, dim3(kGramThreads), smem, st, cube, B, Bp, N, per_cta, s.shift,
+        launch_pdl(kern, grid, dim3(thr), smem, st, cube, B, Bp, N, per_cta, s.shift,
                    s.gram_part, s.sum_part, s.ctl);
     if (ge != cudaSuccess) return ge;
     return launch_reductions(B, N, s.n_part, s, st);
