@@ -1103,10 +1103,11 @@ __device__ __forceinline__ void cp_async_arrive(uint64_t *bar)
 // of the pixels [a, z) of a band row staged at dst; bytes of the cube [lo, hi)
 // only, and nothing past the pixels.
 __device__ __forceinline__ void copy_unit(uint32_t dst, uint64_t a, uint64_t z, uint64_t lo,
-                                          uint64_t hi, uint32_t u, uint64_t pol)
+                                          uint64_t hi, uint32_t u, uint64_t pol, Control *ctl)
 {
     const uint64_t at = (a & ~(uint64_t)15) + 16u * u;
     if (at >= z) return;
+    if (!HSC_IN_BOUNDS(at + 16 > lo && at < hi, ctl)) return;
     if (at >= lo) {
         cp_async16(dst + 16u * u, at, hi - at < 16 ? (uint32_t)(hi - at) : 16u, pol);
     } else {  // a cube that starts inside a unit: its first floats one by one
@@ -1122,7 +1123,7 @@ __device__ __forceinline__ void copy_unit(uint32_t dst, uint64_t a, uint64_t z, 
 // one instruction and one addition each. Pixels at or past N keep what the
 // slot held (the conversion zeroes them).
 __device__ __forceinline__ void fetch_chunk(unsigned char *slot, const float *cube, long N,
-                                            long p0, int B, int t, uint64_t pol)
+                                            long p0, int B, int t, uint64_t pol, Control *ctl)
 {
     constexpr int kStep = kItemCopiers / 16;  // rows between a thread's copies
     const uint32_t base = smem_u32(slot);
@@ -1138,10 +1139,11 @@ __device__ __forceinline__ void fetch_chunk(unsigned char *slot, const float *cu
         uint64_t src = (a & ~(uint64_t)15) + 16u * u;
 #pragma unroll
         for (int i = 0; i < 128 / kStep; ++i) {
-            if ((t >> 4) + i * kStep < B) cp_async16(dst + 16u * u + i * kStep * kItemRow, src, 16u, pol);
+            if ((t >> 4) + i * kStep < B && HSC_IN_BOUNDS(src >= lo && src + 16 <= lo + B * row, ctl))
+                cp_async16(dst + 16u * u + i * kStep * kItemRow, src, 16u, pol);
             src += kStep * row;
         }
-        if (t < B && (a1 & 15) != 0)
+        if (t < B && (a1 & 15) != 0 && HSC_IN_BOUNDS((a1 & ~(uint64_t)15) + 272u <= lo + B * row, ctl))
             cp_async16(dst1 + 256u, (a1 & ~(uint64_t)15) + 256u, 16u, pol);
         return;
     }
@@ -1149,9 +1151,9 @@ __device__ __forceinline__ void fetch_chunk(unsigned char *slot, const float *cu
     const uint64_t n = 4u * (uint64_t)(N - p0 < kChunk ? N - p0 : kChunk);
     for (int i = 0; (t >> 4) + i * kStep < B; ++i) {
         const uint64_t ai = a + (uint64_t)(i * kStep) * row;
-        copy_unit(dst + i * kStep * kItemRow, ai, ai + n, lo, hi, u, pol);
+        copy_unit(dst + i * kStep * kItemRow, ai, ai + n, lo, hi, u, pol, ctl);
     }
-    if (t < B) copy_unit(dst1, a1, a1 + n, lo, hi, 16u, pol);
+    if (t < B) copy_unit(dst1, a1, a1 + n, lo, hi, 16u, pol, ctl);
 }
 
 // A thread's 32 pixels (units u0 .. u0 + kUnits - 1 of 8) of a staged band row
@@ -1343,7 +1345,8 @@ gram_tc_items_kernel(const BatchFrame one, const BatchFrame *__restrict__ frames
                     stop = true;
                     break;
                 }
-                fetch_chunk(staging + slot * kItemStage, fr.cube, fr.N, (long)ch * kChunk, B, t, pol);
+                fetch_chunk(staging + slot * kItemStage, fr.cube, fr.N, (long)ch * kChunk, B, t, pol,
+                            fr.ctl);
                 cp_async_arrive(&bars.full[slot]);
             }
         }

@@ -69,7 +69,7 @@ knn_value_kernel(const float *__restrict__ I, const float *__restrict__ P, int H
     bool bad = false;
     for (int i = tid; i < n2; i += kThreads) {
         unsigned long long e = ~0ull;  // after every entry
-        if (i < n) {
+        if (i < n && HSC_IN_BOUNDS(q0 + i >= 0 && q0 + i < N, ctl)) {
             const float v = I[q0 + i];
             bad |= !isfinite(v);
             e = (unsigned long long)float_to_key(v == 0.f ? 0.f : v) << 32 | (unsigned)(q0 + i);
@@ -154,6 +154,7 @@ knn_value_kernel(const float *__restrict__ I, const float *__restrict__ P, int H
 #pragma unroll
         for (int cl = 0; cl < KC; ++cl) acc[cl] = 0.f;
         for (int a = 0; a < m; ++a) {
+            if (!HSC_IN_BOUNDS(sel[a] >= 0 && sel[a] < N, ctl)) continue;
             const float *Pq = P + sel[a];
 #pragma unroll
             for (int cl = 0; cl < KC; ++cl) acc[cl] += __ldg(Pq + (size_t)cl * (size_t)N);

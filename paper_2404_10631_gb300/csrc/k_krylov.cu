@@ -290,7 +290,9 @@ krylov_kernel(int B, EigFrame fr, const BatchFrame *__restrict__ frames)
                 }
             }
             const int at = (int)rank * kRows + rr;
-            if (df) {
+            if (!HSC_IN_BOUNDS(rr < kRows && at < kPad, fr.ctl)) {
+                // (nothing is written; the barrier below is every thread's)
+            } else if (df) {
                 const dfl w = fast_two_sum(s, lo);
                 if constexpr (CL > 1) store_peer(&sm.x[par][at], (uint32_t)warp, make_float2(w.h, w.l));
                 else sm.x[par][at] = make_float2(w.h, w.l);
@@ -378,6 +380,7 @@ krylov_kernel(int B, EigFrame fr, const BatchFrame *__restrict__ frames)
                 k = j + 1;
                 break;
             }
+            if (!HSC_IN_BOUNDS(j + 1 < kSteps, fr.ctl)) break;  // uniform
             if (tid < kPad) sm.Q[j + 1][tid] = v * ib;
             __syncthreads();
         }

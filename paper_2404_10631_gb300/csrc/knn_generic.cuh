@@ -177,6 +177,7 @@ __device__ __forceinline__ unsigned box_pixel(const TileFrame &f, int p, int K, 
         int cnt = 0;
 #pragma unroll 1
         for (int t = 0; on && t < ntab; t += 8) {  // 8 entries per 16-byte load
+            if (!HSC_IN_BOUNDS(t + 8 <= kTabCap, f.ctl)) break;
             const uint4 w4 = *reinterpret_cast<const uint4 *>(c_knn_tab + t);
             const unsigned w[4] = {w4.x, w4.y, w4.z, w4.w};
             unsigned mask = 0u;
@@ -236,6 +237,7 @@ __device__ __forceinline__ unsigned box_pixel(const TileFrame &f, int p, int K, 
                     const int d = dc + u;
                     in[u] = d >= c0 && d <= c1;
                     if constexpr (kRing) in[u] = in[u] && dr2 + d * d > s0;
+                    in[u] = in[u] && HSC_IN_BOUNDS(q + d >= 0 && q + d < f.N, f.ctl);
                     x[u] = in[u] ? __ldg(Ir + d) : Ip;
                     if constexpr (!kRing)
                         if (in[u]) pv[u].load(Pr, d);
@@ -302,6 +304,7 @@ __device__ __forceinline__ unsigned box_pixel(const TileFrame &f, int p, int K, 
             im = less ? b : im;
         }
         buf.put(im, first);
+        if (!HSC_IN_BOUNDS(im < cap && best.q >= 0 && best.q < f.N, f.ctl)) continue;
         Acc<KC, kP4> x;
         x.load(Acc<KC, kP4>::at(f, best.q), 0);
         acc.add(x);

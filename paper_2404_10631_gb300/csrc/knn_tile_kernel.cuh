@@ -143,6 +143,9 @@ __device__ __forceinline__ bool tile_fast(const TileFrame &f, const TileArgs &a,
                                           int lane, bool on, int vfirst, float l2)
 {
     const int W = f.W, rad = a.rad;
+    // (every access below is within rad of rows r0 .. r0 + kV - 1 and of a
+    // column clamped to rad .. W - 1 - rad)
+    if (!HSC_IN_BOUNDS(r0 >= rad && r0 + kV - 1 + rad < f.H && W > 2 * rad, f.ctl)) return false;
     const int c = c0 + lane;
     // an off lane computes a neighbour's pixel (its loads stay in bounds)
     const int ca = min(max(c, rad), W - 1 - rad);
@@ -228,7 +231,7 @@ __device__ __forceinline__ bool tile_fast(const TileFrame &f, const TileArgs &a,
 #pragma unroll
     for (int i = 0; i < kTileShell; ++i) {
         const char2 d = c_knn_tab[a.disk + min(i, a.shell - 1)];
-        o[i] = d.x * W + d.y;
+        o[i] = HSC_IN_BOUNDS(abs(d.x) <= rad && abs(d.y) <= rad, f.ctl) ? d.x * W + d.y : 0;
     }
     bool bad = false;
     unsigned ord[kV];
@@ -254,6 +257,10 @@ __device__ __forceinline__ bool tile_fast(const TileFrame &f, const TileArgs &a,
             const unsigned i = (ord[v] >> (4 * n)) & 15u;
             const int dr = (int)((a.shell_r >> (4 * i)) & 15u) - 4;
             const int dc = (int)((a.shell_c >> (4 * i)) & 15u) - 4;
+            if (!HSC_IN_BOUNDS(i < (unsigned)a.shell && abs(dr) <= rad && abs(dc) <= rad, f.ctl)) {
+                x[v].zero();
+                continue;
+            }
             x[v].load(Acc<KC, kP4>::at(f, q0 + (v + dr) * W + dc), 0);
         }
 #pragma unroll
@@ -323,7 +330,7 @@ knn_tile_kernel(const __grid_constant__ TileArgs a)
         if (i < g.border_px) {
             int r, c;
             border_pixel(g, f.H, W, a.rad, i, r, c);
-            p0 = r * W + c;
+            if (HSC_IN_BOUNDS(r >= 0 && r < f.H && c >= 0 && c < W, f.ctl)) p0 = r * W + c;
         }
         passes = 1;
     } else {
