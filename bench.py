@@ -9,7 +9,7 @@ lambda = 1, with the library's defaults: the covariance on the tensor cores
 steps are a stream of frames: step i runs on context i % F
 (--frames-in-flight F, default 8; each context has its own CUDA stream,
 scratch and outputs), so while one frame's eigensolver occupies one SM (or,
-for 129-256 bands, its first sweep a cluster of 16) the other frames'
+for 129-256 bands, a cluster of 8) the other frames'
 GPU-wide stages run beside it. "value" is pixels/s over the K
 steps, "latency_ms" the per-frame latency in that stream, "one_in_flight"
 the same steps on one context, and "plain_fp32" the plain per-frame FP32
@@ -494,7 +494,7 @@ def frame_stream(hsc, f, dev, args, world, F, fp32_rate, fp32_peak_note, with_e2
     # ---- the pruned walk's variants (the autotuner's candidates): the KNN
     # stage of the profiled steps per variant, then the tuned variant again
     walk_ms = {}
-    for v in range(6):
+    for v in range(1, 6):  # (0 is 4)
         ctx.set_tuning(B, H, W, k, (tune_cfg["gram_stages"], tune_cfg["svm_px"],
                                     tune_cfg["svm_blocks_per_sm"], v))
         v_ms, _ = profiled()
@@ -502,8 +502,8 @@ def frame_stream(hsc, f, dev, args, world, F, fp32_rate, fp32_peak_note, with_e2
     ctx.set_tuning(B, H, W, k, (tune_cfg["gram_stages"], tune_cfg["svm_px"],
                                 tune_cfg["svm_blocks_per_sm"], tune_cfg["knn_variant"]))
     knn_walks = {"ms_per_launch": {("%d: %s" % (v, name)): round(walk_ms[v], 5)
-                                   for v, name in enumerate(("4 warps", "1 warp", "2 warps", "8 warps",
-                                                             "4 warps", "6 warps"))},
+                                   for v, name in enumerate(("1 warp", "2 warps", "8 warps", "4 warps",
+                                                             "6 warps"), 1)},
                  "tuned": tune_cfg["knn_variant"],
                  "note": "the KNN stage (pruned walk + redo pass) of the profiled steps per walk "
                          "variant; the outputs are the same bit for bit"}

@@ -370,7 +370,7 @@ hsc_status hsc_pca_diagnostics(hsc_ctx *ctx, int32_t *sweeps, int32_t *refine_it
  * thread, the latter meaning 2 with 2 or 3 classes, x 2, 4, 8 or 16 CTAs
  * per SM) and, given KNN parameters with
  * lambda > 0 and the pruned search, of the pruned walk's warps per CTA
- * (variants 0: 4, 1: 1, 2: 2, 3: 8, 4: 4, 5: 6; every pixel's neighbour
+ * (variants 1: 1, 2: 2, 3: 8, 4: 4, 5: 6, 0 as 4; every pixel's neighbour
  * probabilities are added in one
  * canonical order whichever pass completes it, so O is the same) on this cube
  * and model (median of 3 runs each, CUDA events on the context's stream,

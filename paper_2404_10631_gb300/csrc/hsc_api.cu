@@ -563,7 +563,7 @@ hsc_status hsc_autotune(hsc_ctx *ctx, const float *cube, int B, int H, int W,
         // the labels go over the P planes: the walk and its redo pass read the
         // probabilities from the pixel-interleaved copy
         int32_t *lab = reinterpret_cast<int32_t *>(Pm);
-        for (int v = 0; v < hsc::kKnnVariants && err == cudaSuccess; ++v) {
+        for (int v = 1; v < hsc::kKnnVariants && err == cudaSuccess; ++v) {  // (0 is 4)
             const float t = time_ms([&] {
                 return hsc::launch_knn(I, Pm, k, H, W, params->k, params->window_rows,
                                        params->lambda, nullptr, lab, nullptr, s.ctl, str,

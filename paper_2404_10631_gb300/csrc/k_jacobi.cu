@@ -896,8 +896,7 @@ jacobi_kernel(JacParams prm, const double *__restrict__ C, const float2 *__restr
             for (int ii = lane; ii < n; ii += 32)
                 x[ii] = ii < B ? Cp[(size_t)ii * B + j0].x * inv_p2 : 0.f;
         }
-    } else {
-if (presweep) {
+    } else if (presweep) {
         for (int c = warp; c < m; c += nwarps) {
             const float *src = prm.pre + (size_t)c * prm.pre_n;
             float *x = X + (size_t)c * ld;
@@ -961,38 +960,38 @@ if (presweep) {
                 x[b] = oB;
             }
         }
-    } else
-    // a lane's two pairs of a round are disjoint, so both are loaded before
-    // either is stored
-    for (int c = warp; c < m; c += nwarps) {
-        float *x = X + (size_t)c * ld;
-        const int j0 = basis_idx[c];
-        for (int ii = lane; ii < n; ii += 32) x[ii] = (ii == j0) ? 1.f : 0.f;
-        __syncwarp();
-        for (int t = n - 2; t >= 0; --t) {
-            const float2 *lg = rlog + (size_t)t * P;
-            for (int k = lane; k < P; k += 64) {
-                const int k2 = k + 32;
-                const bool has2 = k2 < P;
-                const float2 r1 = lg[k];
-                const float2 r2 = has2 ? lg[k2] : make_float2(1.f, 0.f);
-                int a1, b1, a2 = 0, b2 = 0;
-                pair_ab(t, k, n, a1, b1);
-                if (has2) pair_ab(t, k2, n, a2, b2);
-                const float xa1 = x[a1], xb1 = x[b1];
-                const float xa2 = has2 ? x[a2] : 0.f, xb2 = has2 ? x[b2] : 0.f;
-                if (r1.y != 0.f) {
-                    x[a1] = r1.x * xa1 + r1.y * xb1;
-                    x[b1] = r1.x * xb1 - r1.y * xa1;
-                }
-                if (r2.y != 0.f) {
-                    x[a2] = r2.x * xa2 + r2.y * xb2;
-                    x[b2] = r2.x * xb2 - r2.y * xa2;
-                }
-            }
+    } else {
+        // a lane's two pairs of a round are disjoint, so both are loaded before
+        // either is stored
+        for (int c = warp; c < m; c += nwarps) {
+            float *x = X + (size_t)c * ld;
+            const int j0 = basis_idx[c];
+            for (int ii = lane; ii < n; ii += 32) x[ii] = (ii == j0) ? 1.f : 0.f;
             __syncwarp();
+            for (int t = n - 2; t >= 0; --t) {
+                const float2 *lg = rlog + (size_t)t * P;
+                for (int k = lane; k < P; k += 64) {
+                    const int k2 = k + 32;
+                    const bool has2 = k2 < P;
+                    const float2 r1 = lg[k];
+                    const float2 r2 = has2 ? lg[k2] : make_float2(1.f, 0.f);
+                    int a1, b1, a2 = 0, b2 = 0;
+                    pair_ab(t, k, n, a1, b1);
+                    if (has2) pair_ab(t, k2, n, a2, b2);
+                    const float xa1 = x[a1], xb1 = x[b1];
+                    const float xa2 = has2 ? x[a2] : 0.f, xb2 = has2 ? x[b2] : 0.f;
+                    if (r1.y != 0.f) {
+                        x[a1] = r1.x * xa1 + r1.y * xb1;
+                        x[b1] = r1.x * xb1 - r1.y * xa1;
+                    }
+                    if (r2.y != 0.f) {
+                        x[a2] = r2.x * xa2 + r2.y * xb2;
+                        x[b2] = r2.x * xb2 - r2.y * xa2;
+                    }
+                }
+                __syncwarp();
+            }
         }
-    }
     }
     __syncthreads();
     for (int ii = tid; ii < B; ii += nthr) {  // column 0: the lead

@@ -143,6 +143,12 @@ cudaError_t launch_kc(const float *cube, int B, long N, const float *v1f, const 
                       m ? m->platt_b : nullptr, I_raw, probs, labels, ctl, P4);
 }
 
+// The pixels per thread launch_project_svm and the tuning ask of k classes.
+constexpr bool px_used(int px, int k, bool f64)
+{
+    return px == 1 || (px == 2 ? k == 2 || k == 3 || (f64 ? k == 4 : k == 5) : !f64 && k != 2 && k != 3);
+}
+
 template <int PX, bool kVec, bool kF64>
 cudaError_t dispatch_k(int k, const float *cube, int B, long N, const float *v1f,
                        const float *muf, float *I_raw, const hsc_svm_model *m, float *probs,
@@ -150,13 +156,15 @@ cudaError_t dispatch_k(int k, const float *cube, int B, long N, const float *v1f
 {
     switch (k) {
     case 0:
-        if constexpr (!kF64)
+        if constexpr (!kF64 && px_used(PX, 0, false))
             return launch_kc<0, PX, kVec, false>(cube, B, N, v1f, muf, I_raw, m, probs, labels, ctl, sm, st, mb, P4);
         return cudaErrorInvalidValue;
 #define HSC_SVM_K(KC)                                                                               \
     case KC:                                                                                        \
-        return launch_kc<KC, PX, kVec, kF64>(cube, B, N, v1f, muf, I_raw, m, probs, labels, ctl, sm, \
-                                             st, mb, P4);
+        if constexpr (px_used(PX, KC, kF64))                                                        \
+            return launch_kc<KC, PX, kVec, kF64>(cube, B, N, v1f, muf, I_raw, m, probs, labels, ctl, \
+                                                 sm, st, mb, P4);                                    \
+        return cudaErrorInvalidValue;
         HSC_SVM_K(2)
         HSC_SVM_K(3)
         HSC_SVM_K(4)
@@ -279,7 +287,6 @@ __global__ void __launch_bounds__(kThreads)
 project_multi_kernel(const float *__restrict__ cube, int B, long N, const float *__restrict__ vkf,
                      const float *__restrict__ muf, float *__restrict__ out, Control *ctl)
 {
-    pdl_wait();
     constexpr int S = NP + 1;  // per band: v_0..v_{NP-1}, mu
     extern __shared__ float ws[];
     for (int idx = threadIdx.x; idx < B * S; idx += blockDim.x) {

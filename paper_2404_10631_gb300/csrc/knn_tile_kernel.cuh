@@ -169,7 +169,9 @@ __device__ __forceinline__ bool tile_fast(const TileFrame &f, const TileArgs &a,
         }
         const float L = __fmul_rn(l2, (float)a.sK);
         const float Lp = __fmul_rn(l2, (float)a.prev), Ln = __fmul_rn(l2, (float)a.next);
-        auto decided = [&](float dI) {  // (false for NaN or infinite values)
+        // (false with an infinite value; a NaN neighbour counts as absent, its
+        // own pixel reports it)
+        auto decided = [&](float dI) {
             const float em = __fmul_ru(dI, dI);
             return Ln > __fadd_ru(L, em) && (a.sK == 0 || __fadd_ru(Lp, em) < L);
         };
