@@ -392,7 +392,7 @@ def frame_stream(hsc, f, dev, args, world, F, fp32_rate, fp32_peak_note, with_e2
     tune = {"config": tune_cfg, "seconds": time.perf_counter() - t0,
             "how": "hsc_autotune on the first cube: Gram TMA staging depth {3, 4} (B <= 128), "
                    "projection/SVM {1, 4} pixels per thread x {2, 4, 8, 16} CTAs per SM, pruned "
-                   "KNN walk {4, 1, 2, 8, 4, 6} warps per CTA, "
+                   "KNN walk {1, 2, 8, 4, 6} warps per CTA, "
                    "median of 3 runs each; results do not depend on them"}
     streams = [stream] + [torch.cuda.Stream(dev) for _ in range(F - 1)]
     ctxs = [ctx] + [hsc.Context(dev.index or 0, stream=s) for s in streams[1:]]
@@ -606,7 +606,7 @@ def frame_stream(hsc, f, dev, args, world, F, fp32_rate, fp32_peak_note, with_e2
            "coupling_f64": {"project_svm_ms": f64_ms.get("project_svm"),
                             "project_svm_ms_fp32": stage_ms.get("project_svm"),
                             "frame_ms": sum(f64_ms.values()),
-                            "note": "HSC_SVM_COUPLE_F64: the per-pixel coupling solve in FP64, "
+                            "note": "HSC_SVM_COUPLE_F64: the per-pixel coupling solve to FP64 accuracy, "
                                     "one frame at a time (stage device times)"},
            "roofline": roofline, "stages": stages,
            "knn_full_window": knn_full, "knn_pruned": knn_pruned, "knn_heap": knn_heap,
